@@ -492,7 +492,8 @@ ISPA_API ispa_status ispa_ls_accumulate_ex(ispa_ls_state* state, const void* a_l
 ISPA_API size_t ispa_ls_solve_workspace_size(int32_t dim, int32_t d_out);
 
 /*
- * Closed-form absorption (Eq. 5) and feasibility score (Eq. 6), fp64:
+ * Closed-form absorption (Eq. 5) and feasibility score (Eq. 6), with the accuracy of fp64
+ * arithmetic (products of fp64-grade operands by exact slices on the tensor cores):
  *   dW  = (G + lambda I)^{-1} X W          (Cholesky solve, Eq. 5 with R = Delta W)
  *   eps = || A_loc (W + dW) - A_full W ||_F^2
  *       = tr(W^T S W) - ||L^{-1} X W||_F^2 - lambda ||dW||_F^2,  L L^T = G + lambda I.
@@ -502,7 +503,7 @@ ISPA_API size_t ispa_ls_solve_workspace_size(int32_t dim, int32_t d_out);
  *   eps_out : HOST double (nullable)
  *   lambda  : ridge weight on the unnormalised sums (paper default 1e-3)
  * Synchronises `stream`.  Errors: ISPA_ERR_NOT_SPD if a Cholesky pivot is not
- * positive.
+ * positive (dW and eps are then meaningless); ISPA_ERR_TIMEOUT if a device wait ran out.
  */
 ISPA_API ispa_status ispa_ls_solve(const ispa_ls_state* state, const float* W, int32_t d_out,
                           double lambda, float* dW, double* eps_out, void* workspace,

@@ -1,0 +1,565 @@
+// Products of fp64-grade matrices on the bf16 tensor cores, by exact slices.
+//
+// A number x of a row whose largest magnitude is below 2^E is the fixed-point integer
+// xi = x * 2^(63-E), and xi is split into seven signed 8-bit digits, d_0 .. d_6 in [-128, 128],
+//   x ~= 2^E * sum_p d_p 2^(-7-8p),
+// what is left over being below 2^-56 of the row's largest magnitude (E is the row's own power of
+// two).  A product of two such rows is sum_s 2^(-14-8s) v_s with v_s = sum_{p+q=s} <d_p, d'_q>, s = 0 .. 7
+// (the pairs beyond weigh less than the digits' own remainder; without s = 7 the solve's error, 6e-16 to
+// 2e-15 against 64-bit arithmetic's 5e-16 to 1e-15 on well-conditioned systems, was up to twice as large).  Digits are bf16 numbers,
+// their products integers up to 2^14, and over 128 products of at most 7 pairs a v_s stays below
+// 2^24: the fp32 accumulators of the tensor cores hold it exactly.  So every 128 products the
+// accumulators are read back and added up as 64-bit integers, and a whole contraction is exact
+// but for the digits dropped, in a fixed-point word of 2^-70 of the two rows' scales.  This is the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump (Numer. Algorithms 59, 2012).
+//
+// Why: GB300 has 1.25 TFLOP/s of fp64 against 2250 of dense bf16, so 34 bf16 products for one
+// fp64 product are still an order of magnitude faster.
+//
+// Operand layout ("op").  Rows of a matrix with the contraction index k contiguous, cut into tiles
+// of 64 rows and chunks of 32 k:  [k / 32][row / 64][slice 7][(row / 8) % 8][(k % 32) / 8][row % 8][k % 8]
+// bf16, i.e. 28 KB per (chunk, tile), each 8 x 8 block a 128-byte UMMA core matrix (K-major, no
+// swizzle).  The columns' seven slices arrive by ONE bulk copy, without a tensor map, and slices q,
+// q + 1, ... of it form one operand of 128, 192, ... columns; the rows' come as fourteen copies of 4 KB that put
+// two tiles' slice p together.  So the same op serves as rows (128 of them) and as columns (64).
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "internal.h"
+#include "pdl.cuh"
+#include "ptx.cuh"
+
+namespace ispa {
+
+constexpr int SL = 7;                       // slices
+constexpr int SL_K = 32;                    // k per chunk (one pipeline stage)
+constexpr int SL_BLOCK = 64 * SL_K * 2;     // bytes of 64 rows x 32 k of one slice
+constexpr int SL_TILE = SL * SL_BLOCK;      // of all seven
+constexpr int SL_NAN = 1 << 28;             // exponent of a row that holds a NaN or an infinity
+
+// ---------------------------------------------------------------- digits
+// Fixed-point image of |x| < 2^E with 63 fraction bits, rounded to nearest; integer arithmetic
+// only (the fp64 pipe converts 2 numbers per clock and SM).
+__device__ __forceinline__ int64_t fix63(uint64_t mant, int shift, bool neg) {   // mant * 2^shift
+  uint64_t v;
+  if (shift >= 0) v = mant << shift;
+  else v = shift > -63 ? (mant + (1ull << (-shift - 1))) >> -shift : 0ull;
+  return neg ? -static_cast<int64_t>(v) : static_cast<int64_t>(v);
+}
+
+template <typename T>
+struct SliceSrc;
+template <>
+struct SliceSrc<float> {
+  using Mag = uint32_t;
+  static __device__ Mag mag(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
+  static __device__ int exp_of(Mag m) {
+    const int e = static_cast<int>(m >> 23);
+    return m == 0 ? 0 : (e == 255 ? SL_NAN : e - 126);
+  }
+  static __device__ int64_t fixed(float x, int E) {
+    const uint32_t m = mag(x);
+    const int e = static_cast<int>(m >> 23);
+    const uint64_t mant = (m & 0x7FFFFFu) | (e ? 0x800000u : 0u);
+    return fix63(mant, 63 - E + (e ? e : 1) - 150, __float_as_uint(x) >> 31);
+  }
+};
+template <>
+struct SliceSrc<double> {
+  using Mag = unsigned long long;
+  static __device__ Mag mag(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; }
+  static __device__ int exp_of(Mag m) {
+    const int e = static_cast<int>(m >> 52);
+    return m == 0 ? 0 : (e == 2047 ? SL_NAN : (e ? e - 1022 : -1022));
+  }
+  static __device__ int64_t fixed(double x, int E) {
+    const Mag m = mag(x);
+    const int e = static_cast<int>(m >> 52);
+    const uint64_t mant = (m & 0xFFFFFFFFFFFFFull) | (e ? 1ull << 52 : 0ull);
+    return fix63(mant, 63 - E + (e ? e : 1) - 1075, __double_as_longlong(x) < 0);
+  }
+};
+template <>
+struct SliceSrc<int64_t> {   // fixed point already, 63 fraction bits
+  using Mag = unsigned long long;
+  static __device__ Mag mag(int64_t x) { return x < 0 ? 0ull - static_cast<Mag>(x) : static_cast<Mag>(x); }
+  static __device__ int exp_of(Mag m) { return m == 0 ? 0 : 1 - __clzll(static_cast<long long>(m)); }
+  static __device__ int64_t fixed(int64_t x, int E) { return static_cast<int64_t>(static_cast<uint64_t>(x) << -E); }
+};
+
+// Bytes from an op's start to row r's eight values k .. k + 7 (k % 8 == 0) of slice 0.
+__device__ __forceinline__ int64_t sl_offset(int64_t chunk, int n_t, int r, int kc) {
+  return (chunk * n_t + (r >> 6)) * SL_TILE + ((r >> 3) & 7) * 512 + kc * 128 + (r & 7) * 16;
+}
+
+// The digits of eight fixed-point numbers as bf16, stored at dst + SL_BLOCK * slice (16 bytes each).
+__device__ __forceinline__ void store_digits8(const int64_t* xi, uint8_t* dst) {
+  uint64_t r[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) r[i] = static_cast<uint64_t>(xi[i]);
+#pragma unroll
+  for (int s = 0; s < SL; ++s) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int sh = 56 - 8 * s;
+      // round to nearest without overflow at the top: (r >> (sh - 1) + 1) >> 1
+      const int64_t d = ((static_cast<int64_t>(r[i]) >> (sh - 1)) + 1) >> 1;
+      r[i] -= static_cast<uint64_t>(d) << sh;
+      const uint32_t b = __float_as_uint(static_cast<float>(static_cast<int>(d))) >> 16;   // exact in bf16
+      w[i >> 1] = (i & 1) ? (w[i >> 1] | (b << 16)) : b;
+    }
+    *reinterpret_cast<uint4*>(dst + SL_BLOCK * s) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+struct SliceParams {
+  const void* src;
+  int64_t ld;          // elements between rows (k-contiguous source) or between k (row-contiguous source)
+  int32_t rows, ks;    // valid rows and k of the source (of one segment)
+  int32_t seg_k;       // k of a segment, a multiple of 32 (the padded k when there is one segment)
+  int64_t seg_src;     // elements between the segments' first values in the source
+  int32_t n_t;         // tiles of 64 rows of the op
+  int32_t lower;       // 1: segment z needs the rows above z * seg_k + seg_k - 1 only; -1: the rows below z * seg_k
+  int32_t exp_ld;      // exponents of segment z start at exps + z * exp_ld
+  uint8_t* op;
+  int32_t* exps;
+};
+
+// Source with k contiguous.  One CTA per 8 rows (blockIdx.x) and segment (blockIdx.y): warp w finds row
+// w's exponent, then the warps take the segment's chunks in turn, a thread 8 k of one row, a
+// warp 8 rows x 32 k, so that each slice of it is one contiguous 512-byte store.
+template <typename T>
+__global__ void __launch_bounds__(256) slice_rows_kernel(const SliceParams p) {
+  using S = SliceSrc<T>;
+  pdl_wait();
+  pdl_trigger();
+  __shared__ int e_sh[8];
+  const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r0 = blockIdx.x * 8;
+  if (p.lower > 0 && r0 < (z + 1) * p.seg_k) return;
+  if (p.lower < 0 && r0 >= z * p.seg_k) return;
+  const T* src = static_cast<const T*>(p.src) + z * p.seg_src;
+  typename S::Mag m = 0;
+  if (r0 + warp < p.rows) {
+    const T* row = src + (r0 + warp) * p.ld;
+    for (int k = lane; k < p.ks; k += 32) m = max(m, S::mag(row[k]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) {
+    const int e = S::exp_of(m);
+    e_sh[warp] = e;
+    p.exps[z * p.exp_ld + r0 + warp] = e;
+  }
+  __syncthreads();
+  const int r = lane & 7, kc = lane >> 3;
+  const int E = e_sh[r];
+  const bool live = r0 + r < p.rows && E != SL_NAN;
+  const T* row = src + (r0 + r) * p.ld;
+  for (int c = warp; c < p.seg_k / SL_K; c += 8) {
+    int64_t xi[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int k = c * SL_K + kc * 8 + i;
+      xi[i] = live && k < p.ks ? S::fixed(row[k], E) : 0;
+    }
+    const int64_t ch = static_cast<int64_t>(z) * (p.seg_k / SL_K) + c;
+    store_digits8(xi, p.op + sl_offset(ch, p.n_t, r0 + r, kc));
+  }
+}
+
+// Source with rows contiguous (k strided).  One CTA (8 warps, 32 for long segments) per 32 rows and segment; lane = row, so
+// every load is a contiguous run of the source and every slice store four 128-byte runs.
+template <typename T>
+__global__ void __launch_bounds__(1024) slice_cols_kernel(const SliceParams p) {
+  using S = SliceSrc<T>;
+  pdl_wait();
+  pdl_trigger();
+  __shared__ typename S::Mag red[32][32];
+  const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
+  const int r0 = blockIdx.x * 32, r = r0 + lane;
+  if (p.lower > 0 && r0 < (z + 1) * p.seg_k) return;
+  if (p.lower < 0 && r0 >= z * p.seg_k) return;
+  const T* src = static_cast<const T*>(p.src) + z * p.seg_src + r;
+  const bool in = r < p.rows;
+  typename S::Mag m = 0;
+  if (in) {
+#pragma unroll 8
+    for (int k = warp; k < p.ks; k += n_warp) m = max(m, S::mag(src[k * p.ld]));
+  }
+  red[warp][lane] = m;
+  __syncthreads();
+  for (int w = 0; w < n_warp; ++w) m = max(m, red[w][lane]);
+  const int E = S::exp_of(m);
+  if (r >= p.n_t * 64) return;
+  if (warp == 0) p.exps[z * p.exp_ld + r] = E;
+  const bool live = in && E != SL_NAN;
+  for (int q = warp; q < p.seg_k / 8; q += n_warp) {
+    int64_t xi[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) xi[i] = live && 8 * q + i < p.ks ? S::fixed(src[(8 * q + i) * p.ld], E) : 0;
+    const int64_t ch = static_cast<int64_t>(z) * (p.seg_k / SL_K) + (q >> 2);
+    store_digits8(xi, p.op + sl_offset(ch, p.n_t, r, q & 3));
+  }
+}
+
+// ---------------------------------------------------------------- product
+enum SlMode : int {
+  SL_STORE,   // out[col][row] = product * 2^-row_exp[row]   (row_exp null: 1)
+  SL_SUB,     // out[col][row] -= product
+  SL_CHOL,    // lower tiles: fixed[col][row] -= product, 62 fraction bits
+  SL_DOT      // lower tiles: *dot += sum_{i >= j} (i > j ? 2 : 1) product_ij sym[j][i]
+};
+
+struct SlGemm {
+  const uint8_t* a;       // op of the rows, at its first chunk
+  const uint8_t* b;       // op of the columns
+  int64_t a_chunk, b_chunk;   // bytes between chunks
+  const int32_t* ea;      // exponents of the rows / columns
+  const int32_t* eb;
+  int32_t row0, col0;     // first row and column (multiples of 8)
+  int32_t n_mt, n_nt;     // tiles of 128 rows, of 64 columns (SL_STORE, SL_SUB)
+  int32_t n_tiles;        // all tiles
+  int32_t n_chunks;       // chunks of 32 k
+  int32_t n_split;        // SL_DOT: pieces that the chunks of a tile are cut into (whole flushes); else 1
+  int32_t row_end;        // rows and columns stored stay below these
+  int32_t col_end;
+  int64_t ld;             // elements between columns of out / fixed / rows of sym
+  void* out;
+  const int32_t* row_exp;
+  const float* sym;
+  double* dot;
+  int* status;
+  int* flag;              // bit 1: a device wait ran out
+  uint64_t wait_limit_ns;
+};
+
+constexpr int SG_EPI = 16;             // read-back warps: four per TMEM lane quarter, 16 columns each
+constexpr int SG_COLS = 64 / (SG_EPI / 4);
+constexpr int SG_THREADS = 64 + 32 * SG_EPI;   // warp 0 bulk copies, warp 1 UMMA, then the read-back warps
+constexpr int SG_ST = 2;
+constexpr int SG_A = 2 * SL_TILE;              // 128 rows, [slice][tile]: 56 KB
+constexpr int SG_B = SL_TILE;                  // 64 rows: 28 KB
+constexpr int SG_STAGE = SG_A + SG_B;
+constexpr int SG_OFF_BAR = SG_ST * SG_STAGE;
+constexpr int SG_N_BAR = 2 * SG_ST + 6 + 1;    // stages full / empty, groups full x3 / free x3, drain
+constexpr int SG_S = 8;                        // sums v_0 .. v_7
+// in groups that are read back one after another: s = 0 .. 2, 3 .. 4, 5 .. 7
+__host__ __device__ constexpr int sg_s0(int h) { return h == 0 ? 0 : (h == 1 ? 3 : (h == 2 ? 5 : SG_S)); }
+constexpr int SG_SMEM = SG_OFF_BAR + SG_N_BAR * 8 + 16;
+static_assert(SG_SMEM > 116 * 1024 && SG_SMEM <= 232448, "one CTA per SM");
+constexpr int SG_FLUSH = 4;                    // chunks (128 k) between read-backs: v_s < 2^24
+constexpr uint64_t SG_DRAIN_NS = 200ull * 1000 * 1000;
+
+// K-major operand without swizzle: 128-byte core matrices, `lbo` bytes apart along k, `sbo` along rows.
+__device__ __forceinline__ uint64_t core_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+  return static_cast<uint64_t>((addr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(lbo >> 4) << 16) |
+         (static_cast<uint64_t>(sbo >> 4) << 32) | (1ull << 46);
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
+// (hi 2^32 + lo) 2^e rounded to nearest, without the fp64 pipe (2 operations per clock and SM); e is a row's and a column's exponent and a few tens: normal results only need the
+// integer path, the rest goes through ldexp.
+__device__ __forceinline__ double fixed_to_double(int64_t hi, uint32_t lo, int e) {
+  __int128 v = (static_cast<__int128>(hi) << 32) + lo;
+  const bool neg = v < 0;
+  unsigned __int128 a = neg ? -static_cast<unsigned __int128>(v) : static_cast<unsigned __int128>(v);
+  uint64_t top = static_cast<uint64_t>(a >> 64), low = static_cast<uint64_t>(a);
+  if ((top | low) == 0) return 0.0;
+  int shift = 64;                       // exponent of the word in `top`
+  if (top == 0) {
+    top = low;
+    low = 0;
+    shift = 0;
+  }
+  const int lz = __clzll(static_cast<long long>(top));
+  uint64_t m = lz ? (top << lz) | (low >> (64 - lz)) : top;   // the leading 64 bits
+  const int ex = 1023 + 63 - lz + shift + e;
+  m = (m >> 11) + ((m >> 10) & 1);      // 53 bits; a carry out raises the exponent by itself
+  if (ex < 1 || ex > 2045) return ldexp(neg ? -static_cast<double>(m) : static_cast<double>(m), ex - 1023 - 52);
+  return __longlong_as_double(static_cast<long long>(((static_cast<uint64_t>(ex - 1) << 52) + m) |
+                                                     (neg ? 1ull << 63 : 0ull)));
+}
+
+__device__ __forceinline__ double pow2d(int e) {   // 2^e; 0 below the normal range, inf above it
+  return e < -1022 ? 0.0 : __longlong_as_double(static_cast<long long>(e > 1023 ? 2047 : e + 1023) << 52);
+}
+
+__device__ __forceinline__ void sg_tile(const SlGemm& p, bool tri, int t, int& row, int& col) {
+  if (tri) {   // row tile i holds the 2 (i + 1) column tiles on or below the diagonal
+    int i = static_cast<int>((sqrtf(4.f * t + 1.f) - 1.f) * 0.5f);
+    while (i * (i + 1) > t) --i;
+    while ((i + 1) * (i + 2) <= t) ++i;
+    row = p.row0 + i * 128;
+    col = p.col0 + (t - i * (i + 1)) * 64;
+  } else {   // row tiles vary fastest: the CTAs of a wave share the columns' op
+    row = p.row0 + (t % p.n_mt) * 128;
+    col = p.col0 + (t / p.n_mt) * 64;
+  }
+}
+
+// Work item t: its tile and its chunks [c0, c1).
+__device__ __forceinline__ void sg_item(const SlGemm& p, bool tri, int t, int& row, int& col, int& c0, int& c1) {
+  const int tile = t / p.n_split, piece = t - tile * p.n_split;
+  const int n_flush = (p.n_chunks + SG_FLUSH - 1) / SG_FLUSH;
+  sg_tile(p, tri, tile, row, col);
+  c0 = n_flush * piece / p.n_split * SG_FLUSH;
+  c1 = min(n_flush * (piece + 1) / p.n_split * SG_FLUSH, p.n_chunks);
+}
+
+// 128 x 64 output tiles; TMEM holds the eight v_s of a tile (8 x 64 columns, s after s).  A stage is 32 k
+// of all 14 slices (84 KB), used for all 34 pairs: about 40 bytes per clock of operand traffic, where
+// one pair at a time would need 128.  An UMMA of 128 x 64 x 16 takes as long as one of 128 x 128 x 16 (64
+// clocks, measured), so one slice of the rows meets two or three adjacent slices of the columns in one
+// UMMA of 128 or 192 columns, whose sums are adjacent v_s.
+// The v_s are read back in three groups, each handed over as soon as its last UMMA of the flush is
+// in the stream, so that a read-back runs under the other groups' UMMAs.
+template <int MODE>
+__global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(const SlGemm p) {
+  constexpr bool TRI = MODE == SL_CHOL || MODE == SL_DOT;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SG_OFF_BAR);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + SG_N_BAR);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const uint32_t sbase = smem_u32(smem);
+  const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * SG_ST, gfull0 = empty0 + 8 * SG_ST, gfree0 = gfull0 + 24,
+                 drain_bar = gfree0 + 24;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < SG_ST; ++i) {
+      mbar_init(full0 + 8 * i, 1);
+      mbar_init(empty0 + 8 * i, 1);
+    }
+    for (int i = 0; i < 3; ++i) {
+      mbar_init(gfull0 + 8 * i, 1);
+      mbar_init(gfree0 + 8 * i, SG_EPI);
+    }
+    mbar_init(drain_bar, 1);
+    *abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(tmem_slot), 512);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+  pdl_trigger();
+  const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int g = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x) {
+        int row, col, k0, k1;
+        sg_item(p, TRI, t, row, col, k0, k1);
+        const uint8_t* a = p.a + static_cast<int64_t>(row >> 6) * SL_TILE;
+        const uint8_t* b = p.b + static_cast<int64_t>(col >> 6) * SL_TILE;
+        for (int c = k0; c < k1; ++c, ++g) {
+          const int st = g % SG_ST;
+          if (!mbar_wait(empty0 + 8 * st, ((g / SG_ST) & 1) ^ 1, wc, 41, g)) {
+            ok = false;
+            break;
+          }
+          mbar_arrive_expect_tx(full0 + 8 * st, SG_STAGE);
+          for (int i = 0; i < 2 * SL; ++i)   // slice i >> 1 of row tile i & 1
+            bulk_load(sbase + st * SG_STAGE + i * SL_BLOCK, a + c * p.a_chunk + (i & 1) * SL_TILE + (i >> 1) * SL_BLOCK,
+                      SL_BLOCK, full0 + 8 * st);
+          bulk_load(sbase + st * SG_STAGE + SG_A, b + c * p.b_chunk, SG_B, full0 + 8 * st);
+        }
+      }
+      for (int i = g > SG_ST ? g - SG_ST : 0; i < g; ++i)
+        mbar_wait_drain(full0 + 8 * (i % SG_ST), (i / SG_ST) & 1, SG_DRAIN_NS);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      int g = 0, f = 0;   // stages used, flushes begun
+      bool ok = true;
+      for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x) {
+        int row, col, k0, k1;
+        sg_item(p, TRI, t, row, col, k0, k1);
+        for (int c0 = k0; ok && c0 < k1; c0 += SG_FLUSH, ++f) {
+          const int c1 = min(c0 + SG_FLUSH, k1);
+          for (int c = c0; ok && c < c1; ++c, ++g) {
+            const int st = g % SG_ST;
+            if (!mbar_wait(full0 + 8 * st, (g / SG_ST) & 1, wc, 42, g)) {
+              ok = false;
+              break;
+            }
+            const uint64_t da = core_desc(sbase + st * SG_STAGE, 128, 512);
+            const uint64_t db = core_desc(sbase + st * SG_STAGE + SG_A, 128, 512);
+#pragma unroll
+            for (int h = 0; h < 3; ++h) {
+              // the group's sums of the flush before have been read
+              if (c == c0 && !mbar_wait(gfree0 + 8 * h, (f & 1) ^ 1, wc, 43 + h, f)) {
+                ok = false;
+                break;
+              }
+              tc_fence_after();
+#pragma unroll
+              for (int ks = 0; ks < SL_K / 16; ++ks)
+#pragma unroll
+                for (int i = 0; i < (h < 2 ? sg_s0(h + 1) : SL); ++i) {
+                  // slice q of the rows with the columns' slices s0 .. s1 - 1 in one UMMA: sums q + s0 .. q + s1 - 1.
+                  // The first one of a group starts all of its sums; in the last group that is q = 1 (q = 0 has none for s = 7)
+                  const int q = h == 2 && i < 2 ? 1 - i : i;
+                  const int s0 = sg_s0(h) > q ? sg_s0(h) - q : 0, s1 = sg_s0(h + 1) - q < SL ? sg_s0(h + 1) - q : SL;
+                  umma_ss(tmem + 64 * (q + s0), da + (q * 2 * SL_BLOCK + ks * 256) / 16,
+                          db + (s0 * SL_BLOCK + ks * 256) / 16, idesc_bf16(128, 64 * (s1 - s0), false, false),
+                          (c > c0 || ks > 0 || i > 0) ? 1u : 0u);
+                }
+              if (c == c1 - 1) tc_commit(gfull0 + 8 * h);
+            }
+            if (ok) tc_commit(empty0 + 8 * st);
+          }
+        }
+      }
+      tc_commit(drain_bar);
+      mbar_wait_drain(drain_bar, 0, SG_DRAIN_NS);
+    }
+    __syncwarp();
+  } else {
+    // TMEM lanes 32 quarter .. + 31 (the tile's rows), columns SG_COLS part .. + SG_COLS - 1 of every sum
+    const int quarter = warp & 3, part = (warp - 2) >> 2;
+    const uint32_t tbase = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + SG_COLS * part;
+    double dot = 0.0;
+    int f = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x) {
+      // hi 2^32 + lo, in units of 2^-70 of the rows' scales
+      int64_t hi[SG_COLS];
+      uint32_t lo[SG_COLS];
+#pragma unroll
+      for (int i = 0; i < SG_COLS; ++i) hi[i] = lo[i] = 0;
+      int row, col, k0, k1;
+      sg_item(p, TRI, t, row, col, k0, k1);
+#pragma unroll 1
+      for (int c0 = k0; c0 < k1; c0 += SG_FLUSH, ++f) {
+#pragma unroll
+        for (int h = 0; h < 3; ++h) {
+          ok = ok && __all_sync(0xffffffffu, mbar_wait(gfull0 + 8 * h, f & 1, wc, 46 + h, f));
+          if (!ok) break;
+          tc_fence_after();
+          const int ns = sg_s0(h + 1) - sg_s0(h);
+#pragma unroll
+          for (int c = 0; c < SG_COLS / 8; ++c) {
+            uint32_t v[3][8];
+#pragma unroll
+            for (int s = 0; s < ns; ++s) tmem_ld8(tbase + 64 * (sg_s0(h) + s) + 8 * c, v[s]);
+#pragma unroll
+            for (int s = 0; s < ns; ++s) tmem_wait_ld8(v[s]);
+            if (c == SG_COLS / 8 - 1) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(gfree0 + 8 * h);
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int u0 = __float2int_rn(__uint_as_float(v[0][i])), u1 = __float2int_rn(__uint_as_float(v[1][i]));
+              const int u2 = ns > 2 ? __float2int_rn(__uint_as_float(v[2][i])) : 0;
+              if (h == 0) {
+                hi[8 * c + i] += static_cast<int64_t>(u0 * 256 + u1) * 65536 + static_cast<int64_t>(u2) * 256;   // |u0| <= 2^21
+              } else {
+                if (h == 1) hi[8 * c + i] += u0;
+                const int64_t l = h == 1 ? static_cast<int64_t>(u1) * (1 << 24)
+                                         : static_cast<int64_t>(u0) * 65536 + static_cast<int64_t>(u1) * 256 + u2;
+                const uint64_t sum = static_cast<uint64_t>(lo[8 * c + i]) + static_cast<uint32_t>(l);
+                lo[8 * c + i] = static_cast<uint32_t>(sum);
+                hi[8 * c + i] += (l >> 32) + static_cast<int64_t>(sum >> 32);
+              }
+            }
+          }
+        }
+        if (!ok) break;
+      }
+      if (!ok) break;
+      row += quarter * 32 + lane;
+      col += SG_COLS * part;
+      if (row < p.row_end) {
+        const int ea = p.ea[row];
+        if constexpr (MODE == SL_CHOL) {
+          int64_t* out = static_cast<int64_t*>(p.out) + row;
+#pragma unroll
+          for (int i = 0; i < SG_COLS; ++i) {
+            const int sh = 8 - (ea + p.eb[min(col + i, row)]);   // exponents of factor rows are never above 0
+            hi[i] = sh <= 32 ? static_cast<int64_t>(static_cast<uint64_t>(hi[i]) << (32 - sh)) + (lo[i] >> min(sh, 31) >> (sh == 32))
+                             : hi[i] >> min(sh - 32, 63);
+          }
+          int64_t o[SG_COLS];   // all in flight at once; nothing above the diagonal
+#pragma unroll
+          for (int i = 0; i < SG_COLS; ++i) o[i] = col + i <= row ? out[static_cast<int64_t>(col + i) * p.ld] : 0;
+#pragma unroll
+          for (int i = 0; i < SG_COLS; ++i)
+            if (col + i <= row) out[static_cast<int64_t>(col + i) * p.ld] = o[i] - hi[i];
+        } else {
+          constexpr double kNan = __builtin_nan("");
+          auto value = [&](int i, int c, int de) {   // NaN where the row or the column holds one
+            const int e = ea + p.eb[c];
+            return e > SL_NAN / 2 ? kNan : fixed_to_double(hi[i], lo[i], e - 70 + de);
+          };
+          if constexpr (MODE == SL_DOT) {
+#pragma unroll
+            for (int i = 0; i < SG_COLS; ++i) {
+              const int c = col + i;
+              if (c > row) break;
+              dot = fma(value(i, c, row != c), static_cast<double>(p.sym[static_cast<int64_t>(c) * p.ld + row]), dot);
+            }
+          } else if constexpr (MODE == SL_STORE) {
+            double* out = static_cast<double*>(p.out) + row;
+            const int er = p.row_exp ? p.row_exp[row] : 0;
+#pragma unroll
+            for (int i = 0; i < SG_COLS; ++i)
+              if (col + i < p.col_end) out[static_cast<int64_t>(col + i) * p.ld] = value(i, col + i, -er);
+          } else {
+            double* out = static_cast<double*>(p.out) + row;
+            double x[SG_COLS], o[SG_COLS];
+#pragma unroll
+            for (int i = 0; i < SG_COLS; ++i) x[i] = col + i < p.col_end ? value(i, col + i, 0) : 0.0;
+#pragma unroll
+            for (int i = 0; i < SG_COLS; ++i)   // all in flight at once
+              o[i] = col + i < p.col_end ? out[static_cast<int64_t>(col + i) * p.ld] : 0.0;
+#pragma unroll
+            for (int i = 0; i < SG_COLS; ++i)
+              if (col + i < p.col_end) out[static_cast<int64_t>(col + i) * p.ld] = o[i] - x[i];
+          }
+        }
+      }
+    }
+    if constexpr (MODE == SL_DOT) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+      if (lane == 0) atomicAdd(p.dot, dot);
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag) atomicOr(p.flag, 2);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, 512);
+  }
+}
+
+template <int MODE>
+cudaError_t launch_slice_gemm(const SlGemm& p, int sms, cudaStream_t s) {
+  const cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(slice_gemm_kernel<MODE>), SG_SMEM);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = static_cast<unsigned>(p.n_tiles < sms ? p.n_tiles : sms);
+  return launch_pdl(slice_gemm_kernel<MODE>, dim3(grid), dim3(SG_THREADS), SG_SMEM, s, p);
+}
+
+}  // namespace ispa

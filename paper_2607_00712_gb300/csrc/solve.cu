@@ -1,355 +1,663 @@
-// Closed-form absorption solve (Sec. 3.2, Eq. 5-6) in fp64 on the GPU.
+// Closed-form absorption solve (Sec. 3.2, Eq. 5-6), fp64-grade, on the tensor cores.
 //
 //   M  = G + lambda I                      (G symmetrised from its upper tiles)
-//   L  = chol(M)                           (right-looking blocked Cholesky, NB = 32)
-//   Y  = L^{-1} (X W)                      (blocked forward substitution)
-//   dW = L^{-T} Y                          (blocked back substitution)
+//   L  = chol(M)                           (right-looking, panels of 64 columns)
+//   Y  = L^{-1} (X W)                      (forward substitution in blocks of 128 rows)
+//   dW = L^{-T} Y                          (back substitution)
 //   eps = tr(W^T S W) - ||Y||_F^2 - lambda ||dW||_F^2
 // The eps expression is Eq. 6 expanded with the normal equations
 // (G + lambda I) dW = X W, which give tr(dW^T G dW) = ||Y||^2 - lambda||dW||^2
-// and tr(dW^T X W) = ||Y||^2.  It runs once per layer at the transition, so
-// the kernels are plain fp64 SIMT code bounded by GB300's fp64 rate.
+// and tr(dW^T X W) = ||Y||^2.
+//
+// Every cubic part is a product, and every product goes through slicemm.cuh (34 exact bf16 products
+// for one fp64 one): X W, the trailing updates of the factorisation and of both substitutions, the
+// products with the inverses of L's 128 x 128 diagonal blocks, and tr(W^T S W) = sum_ij S_ij (W W^T)_ij, half
+// the work of S W and nothing to store.  Plain fp64 code ran all of it at 1.09 TFLOP/s, the chip's
+// fp64 rate: 782 ms at hidden 5120 and 33 ms at 1536 (where the panels' launches and latency counted
+// too), against 30.5 and 3.1 ms.  What bounds it now: at 5120 the products' tensor time and read-back (24
+// of 30 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
+// dW's error against 64-bit arithmetic (before its rounding to fp32) is 0.4 to 0.8 times the plain code's.
+//
+// The factorisation runs in fixed point.  Row and column i are scaled by a power of two (exactly)
+// so that M_ii lies in [1/4, 1); then every |M_ij|, every element of every Schur complement and
+// every |L_ij| of a positive definite M is below 1, and 64-bit words with 62 (M) and 63 (L) fraction bits
+// hold them with an absolute error of 2^-62, where fp64 has 2^-54 near 1.  The trailing update is then
+// an integer subtraction, and a panel runs on the integer pipe.  A word that leaves its range shows
+// that M is not positive definite, like a pivot that isn't positive.
+//
+// All of it is stored by columns (element (i, j) at [j][i]): a tile's epilogue thread owns a row,
+// so its warp's accesses run along a column.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "internal.h"
-#include "ptx.cuh"
+#include "slicemm.cuh"
 
 namespace ispa {
 
 namespace {
 
-constexpr int NB = 32;    // Cholesky / triangular block
-constexpr int TB = 64;    // GEMM tile
-constexpr int TK = 16;    // GEMM k step
+constexpr int NB = 64;     // panel of the factorisation
+constexpr int TB = 128;    // block of the substitutions
+constexpr int PR = 32;     // panel rows per CTA
+constexpr int FLAG_NOT_SPD = 1;
 
-enum MatMode : int { M_F32 = 0, M_F64 = 1, M_F64_T = 2, M_F32_SYM = 3 };
+// t_i: the power of two with M_ii 2^(-2 t_i) in [1/4, 1).  Rows past D (padding) get 0.
+__global__ void __launch_bounds__(256) equil_kernel(const float* __restrict__ gram, int D, int Dp, double lambda,
+                                                    int32_t* __restrict__ t, int* flag) {
+  pdl_wait();
+  pdl_trigger();
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= Dp) return;
+  int e = 0;
+  if (i < D) {
+    const double v = static_cast<double>(gram[static_cast<int64_t>(i) * (2 * D) + i]) + lambda;
+    if (v > 0.0 && v <= 1.7976931348623157e308) {
+      e = (SliceSrc<double>::exp_of(SliceSrc<double>::mag(v)) + 1) >> 1;
+    } else {
+      atomicOr(flag, FLAG_NOT_SPD);
+    }
+  }
+  t[i] = e;
+}
 
-struct MatRef {
-  const void* p;
-  int64_t ld;
-  int mode;
+// fix[j][i] (i >= j) = M_ij 2^(-t_i - t_j) with 62 fraction bits, from G's upper triangle (row j of G is column
+// j here); the padding is the identity / 2.
+__global__ void __launch_bounds__(256) form_kernel(const float* __restrict__ gram, int D, int Dp, double lambda,
+                                                   const int32_t* __restrict__ t, int64_t* __restrict__ fix, int* flag) {
+  pdl_wait();
+  pdl_trigger();
+  const int j = blockIdx.x;
+  const int i = blockIdx.y * 256 + threadIdx.x;
+  if (i < j || i >= Dp) return;
+  int64_t v = 0;
+  if (i >= D) {
+    v = i == j ? int64_t{1} << 61 : 0;
+  } else {
+    const float g = gram[static_cast<int64_t>(j) * (2 * D) + i];
+    const int e = t[i] + t[j];
+    bool bad;
+    if (i == j) {
+      const double d = static_cast<double>(g) + lambda;
+      bad = !(d > 0.0 && d <= 1.7976931348623157e308);
+      v = bad ? int64_t{1} << 61 : SliceSrc<double>::fixed(d, e + 1);
+    } else {
+      const uint32_t m = SliceSrc<float>::mag(g);
+      const int ge = SliceSrc<float>::exp_of(m);   // |g| < 2^ge
+      bad = m != 0 && ge - e > 1;                  // |M_ij| >= 1 (or not finite): not positive definite
+      if (!bad && m != 0) {
+        v = SliceSrc<float>::fixed(g, e + 1);
+        bad = v >= (int64_t{1} << 62) || v <= -(int64_t{1} << 62);
+      }
+      if (bad) v = 0;
+    }
+    if (bad) atomicOr(flag, FLAG_NOT_SPD);
+  }
+  fix[static_cast<int64_t>(j) * Dp + i] = v;
+}
+
+// 1 / sqrt of the pivot d (62 fraction bits): y 2^e, y in [1, 2] with 62 fraction bits.  The fp32
+// estimate m 2^-23 and one third-order Newton step in fixed point: y += y (err / 2 + 3/8 err^2),
+// err = 1 - v y^2 below 2^-21.
+__device__ __forceinline__ void pivot_rsqrt(int64_t d, uint64_t& y, int& e) {
+  const int s = __clzll(d) & ~1;
+  const uint64_t u = static_cast<uint64_t>(d) << s;   // v = u 2^-64 in [1/4, 1), d = v 2^(2 - s)
+  e = (s - 2) >> 1;
+  const float v = __uint2float_rn(static_cast<uint32_t>(u >> 32));
+  float yf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(v));   // 2^-16 v^(-1/2)
+  const uint32_t m = min(max(__float2uint_rn(yf * 549755813888.f), 1u << 23), 1u << 24);   // 2^39
+  const uint64_t t = __umul64hi(u, static_cast<uint64_t>(m) * m << 14);   // v y^2, 60 fraction bits
+  const int64_t err = static_cast<int64_t>((1ull << 60) - t);
+  const int e20 = static_cast<int>(err >> 20);
+  const int64_t corr = (err >> 1) + ((3 * ((static_cast<int64_t>(e20) * e20) >> 20)) >> 3);
+  y = (static_cast<uint64_t>(m) << 39) + static_cast<uint64_t>((static_cast<int64_t>(m) * corr) >> 21);
+}
+
+// c (62 fraction bits) times y 2^e with 63 fraction bits; a magnitude of 1 or more sets `over`.
+__device__ __forceinline__ int64_t scale_col(int64_t c, uint64_t y, int e, bool& over) {
+  const int64_t c1 = static_cast<int64_t>(static_cast<uint64_t>(c) << (e + 1));
+  const __int128 p = static_cast<__int128>(c1) * static_cast<int64_t>(y >> 1);
+  const int64_t hi = static_cast<int64_t>(p >> 64);
+  over |= (c1 >> (e + 1)) != c || static_cast<uint64_t>(hi + (int64_t{1} << 60)) >= (uint64_t{1} << 61);
+  return static_cast<int64_t>(p >> 61);
+}
+
+struct PanelParams {
+  int64_t* fix;       // [Dp][Dp] by columns: M, overwritten by L below the diagonal blocks
+  int64_t* diag;      // [Dp / 64][64][64] by columns: L of the diagonal blocks
+  int32_t Dp, k0;
+  uint8_t* op;        // slices of the panel's rows (2 chunks of 32 columns)
+  int32_t n_t;
+  int32_t* exps;      // their exponents
+  int* flag;
+  int* status;
+  uint64_t wait_limit_ns;
 };
 
-__device__ __forceinline__ double mat_get(const MatRef& m, int64_t i, int64_t k) {
-  switch (m.mode) {
-    case M_F32: return static_cast<double>(static_cast<const float*>(m.p)[i * m.ld + k]);
-    case M_F64: return static_cast<const double*>(m.p)[i * m.ld + k];
-    case M_F64_T: return static_cast<const double*>(m.p)[k * m.ld + i];
-    default: {
-      const int64_t a = i < k ? i : k, b = i < k ? k : i;
-      return static_cast<double>(static_cast<const float*>(m.p)[a * m.ld + b]);
-    }
-  }
+// Elements of L as the panel's dot products take them: the high word of the 63 fraction bits and the
+// next 27 bits.  A multiply-add is then three 32 x 32 + 64 bit ones without any shift or carry (a 64-bit
+// multiply-high takes 21 issue slots, these 12); the middle sums of 64 products of rows whose norm is at most 1
+// stay below 2^63.  What is dropped is below 2^-58 of the other factor a term, where fp64 rounds the
+// running sum to 2^-54 of itself.
+__device__ __forceinline__ int2 pack_l(int64_t l) {
+  return make_int2(static_cast<int>(l >> 32), static_cast<int>(static_cast<uint32_t>(l) >> 5));
 }
-
-// C[M][N] = alpha * A[M][K] B[K][N] + beta * C (fp64).  lower_only skips tiles
-// strictly above the diagonal of C.
-__global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, MatRef A, MatRef B, double* C,
-                                                    int64_t ldc, double alpha, double beta,
-                                                    int lower_only) {
-  const int bx = blockIdx.x, by = blockIdx.y;
-  if (lower_only && bx * TB > by * TB + TB - 1) return;
-  __shared__ double As[TK][TB + 1];
-  __shared__ double Bs[TK][TB + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
-  const int row0 = by * TB, col0 = bx * TB;
-  for (int k0 = 0; k0 < K; k0 += TK) {
-    for (int e = threadIdx.x; e < TK * TB; e += 256) {
-      const int kk = e / TB, ii = e % TB;
-      const int gi = row0 + ii, gk = k0 + kk;
-      As[kk][ii] = (gi < M && gk < K) ? mat_get(A, gi, gk) : 0.0;
-      const int gj = col0 + ii;
-      Bs[kk][ii] = (gk < K && gj < N) ? mat_get(B, gk, gj) : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < TK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fma(a[r], b[c], acc[r][c]);
-    }
-    __syncthreads();
+struct Dot {
+  int64_t hi = 0, mid = 0;
+  __device__ __forceinline__ void add(const int2 a, const int2 b) {
+    hi += static_cast<int64_t>(a.x) * b.x;
+    mid += static_cast<int64_t>(a.x) * b.y;
+    mid += static_cast<int64_t>(a.y) * b.x;
   }
+  __device__ __forceinline__ int64_t sum() const { return hi + (mid >> 27); }   // 62 fraction bits
+};
+
+// One panel: every CTA factors the 64 x 64 diagonal block for itself (the same work on every SM, and
+// no launch between it and the rows that need it) together with 32 rows below it, whose slices it writes.
+// Column by column, four lanes a row (k mod 4 of its dot product).  What bounds it is the chain of the
+// diagonal block's 64 columns: l of the last column -> the pivot and its reciprocal root -> the column's
+// scaling.  So one warp keeps the diagonal up to date and does nothing but pivots, two scale, and eight take
+// the next column's dot products, all but their last term, in the meantime.  The rows below the block
+// aren't on the chain: their four warps follow at their own pace, an mbarrier per column.  (All rows in step
+// took 1800 clocks a column, 63 us a panel, and one right-looking column at a time 3900.)
+constexpr int PROWS = NB + PR;          // rows in shared memory
+constexpr int PLD = NB + 1;
+constexpr int PL = 4;                   // lanes per row
+constexpr int P_DOT = PL * NB;          // threads of the diagonal block's dot products,
+constexpr int P_SCALE = P_DOT + NB;     // its scaling up to here,
+constexpr int P_CHAIN = P_SCALE + 32;   // the pivots' warp up to here,
+constexpr int P_THREADS = P_CHAIN + PL * PR;   // and the rows below
+constexpr int PANEL_SMEM = (2 * PROWS * PLD + 3 * NB) * 8 + NB * 4 + 16;
+static_assert(P_THREADS <= 1024, "panel roles");
+__device__ __forceinline__ void chain_sync() { asm volatile("bar.sync 1, %0;" ::"n"(P_CHAIN) : "memory"); }
+
+__global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
+  extern __shared__ int64_t psm[];
+  int64_t* a = psm;                                               // [row][PLD]: M, then L
+  int2* pk = reinterpret_cast<int2*>(psm + PROWS * PLD);           // L for the dot products
+  uint64_t* ys = reinterpret_cast<uint64_t*>(psm + 2 * PROWS * PLD);   // the pivots' reciprocal roots
+  int64_t* cs = reinterpret_cast<int64_t*>(ys + NB);               // column j before its scaling
+  uint64_t* done = reinterpret_cast<uint64_t*>(cs + NB);           // mbarrier j: column j of the diagonal block is complete
+  int* es = reinterpret_cast<int*>(done + NB);
+  volatile int* abort_flag = es + NB;
+  pdl_wait();
+  pdl_trigger();
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int r0 = p.k0 + NB + blockIdx.x * PR;   // this CTA's first row below the diagonal block
+  const bool rows = r0 < p.Dp;
+  bool over = false;   // a pivot that isn't positive, or an element of L not below 1: not positive definite
+  {
+    const int64_t* col0 = p.fix + static_cast<int64_t>(p.k0) * p.Dp;
+    // all of a thread's loads in flight at once
+    constexpr int ND = (NB * NB + P_THREADS - 1) / P_THREADS, NX = (NB * PR + P_THREADS - 1) / P_THREADS;
+    int64_t d[ND], x[NX];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int gi = row0 + ty + 16 * r;
-    if (gi >= M) continue;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int gj = col0 + tx + 16 * c;
-      if (gj >= N) continue;
-      double* cp = C + gi * ldc + gj;
-      *cp = alpha * acc[r][c] + (beta == 0.0 ? 0.0 : beta * *cp);
+    for (int i = 0; i < ND; ++i) {
+      const int e = tid + i * P_THREADS, c = e >> 6, r = e & 63;
+      d[i] = e < NB * NB && r >= c ? col0[static_cast<int64_t>(c) * p.Dp + p.k0 + r] : 0;
     }
-  }
-}
-
-// M = sym(G) + lambda I, fp64 [D][D].  G's upper triangle is always valid.
-__global__ void form_spd_kernel(const float* __restrict__ gram, int D, double lambda, double* __restrict__ L) {
-  const int64_t n = static_cast<int64_t>(D) * D;
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const int i = static_cast<int>(e / D), j = static_cast<int>(e % D);
-    const int a = i < j ? i : j, b = i < j ? j : i;
-    double v = static_cast<double>(gram[static_cast<int64_t>(a) * (2 * D) + b]);
-    if (i == j) v += lambda;
-    L[e] = v;
-  }
-}
-
-// Unblocked Cholesky of the nb x nb diagonal block at (k0, k0), in place (lower).
-__global__ void __launch_bounds__(256) potrf_diag_kernel(double* L, int D, int k0, int nb, int* flag) {
-  __shared__ double a[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    a[i][j] = L[static_cast<int64_t>(k0 + i) * D + k0 + j];
+#pragma unroll
+    for (int i = 0; i < NX; ++i) {
+      const int e = tid + i * P_THREADS;
+      x[i] = e < NB * PR && rows ? col0[static_cast<int64_t>(e >> 5) * p.Dp + r0 + (e & 31)] : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < ND; ++i) {
+      const int e = tid + i * P_THREADS;
+      if (e < NB * NB) a[(e & 63) * PLD + (e >> 6)] = d[i];
+    }
+#pragma unroll
+    for (int i = 0; i < NX; ++i) {
+      const int e = tid + i * P_THREADS;
+      if (e < NB * PR) a[(NB + (e & 31)) * PLD + (e >> 5)] = x[i];
+    }
+    if (tid < NB) mbar_init(smem_u32(done + tid), 1);
+    if (tid == 0) *abort_flag = 0;
   }
   __syncthreads();
-  for (int j = 0; j < nb; ++j) {
-    if (threadIdx.x == 0) {
-      double d = a[j][j];
-      if (!(d > 0.0)) {
-        atomicExch(flag, 1);
-        d = 1.0;  // keep the remaining arithmetic finite; the caller reports NOT_SPD
+  if (tid < P_DOT) {
+    const int r = tid / PL, h = tid % PL;
+    const int2* row = pk + r * PLD;
+    Dot acc;              // this lane's share of column j's dot product
+    const int first = (tid >> 5) * (32 / PL);   // the warp's first row
+#pragma unroll 1
+    for (int j = 0; j < NB; ++j) {
+      Dot next;
+      if (r > j) {
+        if (j > 0 && (j - 1) % PL == h) acc.add(row[j - 1], pk[j * PLD + j - 1]);
+        const int past = PL * (j + 1 - first);   // lanes of the rows up to j
+        const unsigned live = past > 0 ? 0xFFFFFFFFu << past : 0xFFFFFFFFu;
+        int64_t sum = acc.sum();
+#pragma unroll
+        for (int o = PL / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(live, sum, o);
+        if (h == 0) cs[r] = a[r * PLD + j] - sum;
+        if (j + 1 < NB) {
+          const int2* ln = pk + (j + 1) * PLD;
+#pragma unroll 4
+          for (int k = h; k < j; k += PL) next.add(row[k], ln[k]);
+        }
       }
-      a[j][j] = sqrt(d);
+      acc = next;
+      chain_sync();   // pivot j
+      chain_sync();   // column j
     }
-    __syncthreads();
-    for (int i = j + 1 + threadIdx.x; i < nb; i += blockDim.x) a[i][j] /= a[j][j];
-    __syncthreads();
-    const int m = nb - j - 1;
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-      const int i = j + 1 + e / m, k = j + 1 + e % m;
-      if (k <= i) a[i][k] -= a[i][j] * a[k][j];
+  } else if (tid < P_SCALE) {
+    const int r = tid - P_DOT;
+#pragma unroll 1
+    for (int j = 0; j < NB; ++j) {
+      chain_sync();   // pivot j
+      if (r > j) {
+        const int64_t l = scale_col(cs[r], ys[j], es[j], over);
+        pk[r * PLD + j] = pack_l(l);
+        a[r * PLD + j] = l;
+      }
+      chain_sync();   // column j
     }
-    __syncthreads();
-  }
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    L[static_cast<int64_t>(k0 + i) * D + k0 + j] = j <= i ? a[i][j] : 0.0;
-  }
-}
-
-// Panel: rows i >= k0+nb solve x L11^T = a (one row per thread).
-__global__ void __launch_bounds__(128) trsm_panel_kernel(double* L, int D, int k0, int nb) {
-  __shared__ double l11[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    l11[i][j] = L[static_cast<int64_t>(k0 + i) * D + k0 + j];
+  } else if (tid < P_CHAIN) {
+    int64_t d0 = a[lane * PLD + lane], d1 = a[(lane + 32) * PLD + lane + 32];   // diagonal elements lane, lane + 32
+#pragma unroll 1
+    for (int j = 0; j < NB; ++j) {
+      if (j > 0) {
+        Dot q0, q1;
+        const int2 l0 = pk[lane * PLD + j - 1], l1 = pk[(lane + 32) * PLD + j - 1];
+        q0.add(l0, l0);
+        q1.add(l1, l1);
+        d0 -= lane >= j ? q0.sum() : 0;
+        d1 -= lane + 32 >= j ? q1.sum() : 0;
+      }
+      int64_t d = __shfl_sync(0xffffffffu, j < 32 ? d0 : d1, j & 31);
+      if (d <= 0) {
+        over = true;
+        d = int64_t{1} << 61;   // keep the remaining arithmetic in range; the caller reports NOT_SPD
+      }
+      uint64_t y;
+      int e;
+      pivot_rsqrt(d, y, e);
+      if (lane == 0) {
+        ys[j] = y;
+        es[j] = e;
+      }
+      chain_sync();   // pivot j
+      // sqrt(d) = d / sqrt(d); the chain reads no diagonal element of L
+      if (lane == 0) a[j * PLD + j] = static_cast<int64_t>((static_cast<__int128>(d) * y) >> (61 - e));
+      chain_sync();   // column j
+      if (lane == 0) mbar_arrive(smem_u32(done + j));
+    }
+  } else {
+    const int t = tid - P_CHAIN, h = t % PL, r = NB + t / PL;
+    int2* row = pk + r * PLD;
+    const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
+#pragma unroll 1
+    for (int j = 0; j < NB; ++j) {
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(done + j), 0, wc, 61, j))) break;
+      const int2* ln = pk + j * PLD;
+      Dot acc;
+#pragma unroll 4
+      for (int k = h; k < j; k += PL) acc.add(row[k], ln[k]);
+      int64_t sum = acc.sum();
+#pragma unroll
+      for (int o = PL / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      const int64_t l = scale_col(a[r * PLD + j] - sum, ys[j], es[j], over);
+      __syncwarp();
+      if (h == 0) {
+        row[j] = pack_l(l);
+        a[r * PLD + j] = l;
+      }
+      __syncwarp();
+    }
   }
   __syncthreads();
-  const int i = k0 + nb + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= D) return;
-  double* row = L + static_cast<int64_t>(i) * D + k0;
-  double x[NB];
-#pragma unroll
-  for (int j = 0; j < NB; ++j) {
-    if (j < nb) {
-      double v = row[j];
-      for (int m = 0; m < j; ++m) v -= x[m] * l11[j][m];
-      x[j] = v / l11[j][j];
-    }
+  if (tid == 0 && *abort_flag) atomicOr(p.flag, 2);
+  if (over) atomicOr(p.flag, FLAG_NOT_SPD);
+  if (blockIdx.x == 0) {
+    int64_t* dst = p.diag + static_cast<int64_t>(p.k0 / NB) * (NB * NB);   // by columns
+    for (int e = tid; e < NB * NB; e += P_THREADS) dst[e] = (e & 63) >= (e >> 6) ? a[(e & 63) * PLD + (e >> 6)] : 0;
   }
+  if (!rows) return;
+  for (int e = tid; e < NB * PR; e += P_THREADS)
+    p.fix[static_cast<int64_t>(p.k0 + (e >> 5)) * p.Dp + r0 + (e & 31)] = a[(NB + (e & 31)) * PLD + (e >> 5)];
+  if (tid < 256) {
+    // slices: warp w takes the 8 columns 8 w .. of the 32 rows; a row's exponent from all 64
+    const int kc = tid >> 5;
+    const int64_t* row = a + (NB + lane) * PLD;
+    uint64_t mx = 0;
+#pragma unroll 16
+    for (int k = 0; k < NB; ++k) mx |= static_cast<uint64_t>(SliceSrc<int64_t>::mag(row[k]));   // same leading bit as the maximum
+    const int E = SliceSrc<int64_t>::exp_of(mx);
+    if (kc == 0) p.exps[r0 + lane] = E;
+    int64_t xi[8];
 #pragma unroll
-  for (int j = 0; j < NB; ++j)
-    if (j < nb) row[j] = x[j];
+    for (int i = 0; i < 8; ++i) xi[i] = SliceSrc<int64_t>::fixed(row[kc * 8 + i], E);
+    store_digits8(xi, p.op + sl_offset(kc >> 2, p.n_t, r0 + lane, kc & 3));
+  }
 }
 
-// Forward block: L11 Y1 = B1 for rows k0..k0+nb (one column of B per thread).
-__global__ void trsv_fwd_kernel(const double* L, int D, int k0, int nb, double* B, int n_cols) {
-  __shared__ double l11[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    l11[i][j] = L[static_cast<int64_t>(k0 + i) * D + k0 + j];
+// Inverse of L's 128 x 128 diagonal blocks, fp64: inv[b][i][j] and its transpose.  One CTA per 8
+// columns of a block; thread (column, row group): right-looking substitution with its rows in registers.
+constexpr int IC = 8;
+constexpr int IG = 256 / IC;   // row groups
+constexpr int INV_SMEM = (TB * (TB + 1) + 2 * IC + TB) * 8;
+__global__ void __launch_bounds__(256) inverse_kernel(const int64_t* __restrict__ fix, const int64_t* __restrict__ diag,
+                                                      int Dp, double* __restrict__ inv, double* __restrict__ inv_t) {
+  extern __shared__ double sm[];
+  double* l = sm;                        // by columns, [c][TB + 1]
+  double* xs = sm + TB * (TB + 1);       // the current row of the solution, twice
+  double* rd = xs + 2 * IC;                  // reciprocals of the diagonal
+  pdl_wait();
+  pdl_trigger();
+  const int b = blockIdx.y, c0 = blockIdx.x * IC, tid = threadIdx.x;
+  constexpr double k63 = 1.0842021724855044e-19;   // 2^-63
+  for (int e = tid; e < TB * TB; e += 256) {
+    const int c = e >> 7, r = e & 127;
+    if (r < c) continue;
+    int64_t v;
+    if ((c >> 6) == (r >> 6)) v = diag[(static_cast<int64_t>(2 * b + (c >> 6)) << 12) + ((c & 63) << 6) + (r & 63)];
+    else v = fix[static_cast<int64_t>(b * TB + c) * Dp + b * TB + r];
+    const double d = static_cast<double>(v) * k63;
+    l[c * (TB + 1) + r] = d;
+    if (c == r) rd[c] = 1.0 / d;
   }
   __syncthreads();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_cols) return;
-  double y[NB];
+  const int col = tid % IC, g = tid / IC;
+  double x[TB / IG];
 #pragma unroll
-  for (int i = 0; i < NB; ++i) {
-    if (i < nb) {
-      double v = B[static_cast<int64_t>(k0 + i) * n_cols + c];
-      for (int m = 0; m < i; ++m) v -= l11[i][m] * y[m];
-      y[i] = v / l11[i][i];
-      B[static_cast<int64_t>(k0 + i) * n_cols + c] = y[i];
+  for (int m = 0; m < TB / IG; ++m) x[m] = g + IG * m == c0 + col ? 1.0 : 0.0;
+#pragma unroll
+  for (int k = 0; k < TB; ++k) {
+    if (k < c0) continue;
+    double* xk = xs + (k & 1) * IC;   // alternating: one barrier a step
+    if (g == k % IG) {
+      x[k / IG] *= rd[k];
+      xk[col] = x[k / IG];
     }
+    __syncthreads();
+    const double v = xk[col];
+#pragma unroll
+    for (int m = k / IG; m < TB / IG; ++m)
+      if (g + IG * m > k) x[m] = fma(-l[k * (TB + 1) + g + IG * m], v, x[m]);
+  }
+  const int64_t base = static_cast<int64_t>(b) * TB * TB;
+#pragma unroll
+  for (int m = 0; m < TB / IG; ++m) {
+    const int i = g + IG * m, j = c0 + col;
+    const double v = i >= j ? x[m] : 0.0;
+    inv[base + i * TB + j] = v;
+    inv_t[base + j * TB + i] = v;
   }
 }
 
-// Backward block: L11^T Z1 = Y1 for rows k0..k0+nb.
-__global__ void trsv_bwd_kernel(const double* L, int D, int k0, int nb, double* B, int n_cols) {
-  __shared__ double l11[NB][NB + 1];
-  for (int e = threadIdx.x; e < nb * nb; e += blockDim.x) {
-    const int i = e / nb, j = e % nb;
-    l11[i][j] = L[static_cast<int64_t>(k0 + i) * D + k0 + j];
-  }
-  __syncthreads();
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_cols) return;
-  double z[NB];
-#pragma unroll
-  for (int i = NB - 1; i >= 0; --i) {
-    if (i < nb) {
-      double v = B[static_cast<int64_t>(k0 + i) * n_cols + c];
-      for (int m = i + 1; m < nb; ++m) v -= l11[m][i] * z[m];
-      z[i] = v / l11[i][i];
-      B[static_cast<int64_t>(k0 + i) * n_cols + c] = z[i];
-    }
-  }
-}
-
-// out += sum_e x[e] * y[e]  (y of type float or double; y == nullptr means y = x)
-template <typename TY>
-__global__ void __launch_bounds__(256) dot_kernel(const double* __restrict__ x, const TY* __restrict__ y,
-                                                  int64_t n, double* out) {
-  double s = 0.0;
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    s += x[e] * (y ? static_cast<double>(y[e]) : x[e]);
+// *out += sum x^2
+__device__ __forceinline__ void block_add(double s, double* out) {
   __shared__ double red[8];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
+  if (threadIdx.x == 0) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) atomicAdd(out, s);
+    for (int i = 1; i < 8; ++i) s += red[i];
+    atomicAdd(out, s);
   }
 }
 
-__global__ void to_f32_kernel(const double* __restrict__ x, float* __restrict__ y, int64_t n) {
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; e < n;
-       e += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    y[e] = static_cast<float>(x[e]);
+__global__ void __launch_bounds__(256) sumsq_kernel(const double* __restrict__ x, int64_t n, double* out) {
+  pdl_wait();
+  pdl_trigger();
+  double s = 0.0;
+  for (int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; e < n; e += static_cast<int64_t>(gridDim.x) * 256)
+    s = fma(x[e], x[e], s);
+  block_add(s, out);
+}
+
+// dW[i][j] = z[j][i] 2^(-t_i), through 32 x 32 tiles; *out += ||dW||^2 (before the fp32 rounding).
+__global__ void __launch_bounds__(256) finish_kernel(const double* __restrict__ z, int D, int Dp, int n,
+                                                     const int32_t* __restrict__ t, float* __restrict__ dW, double* out) {
+  __shared__ float tile[32][33];
+  pdl_wait();
+  pdl_trigger();
+  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double s = 0.0;
+  for (int jj = w; jj < 32; jj += 8) {
+    double v = 0.0;
+    if (j0 + jj < n && i0 + lane < D) v = z[static_cast<int64_t>(j0 + jj) * Dp + i0 + lane] * pow2d(-t[i0 + lane]);
+    s = fma(v, v, s);
+    tile[jj][lane] = static_cast<float>(v);
+  }
+  __syncthreads();
+  for (int ii = w; ii < 32; ii += 8)
+    if (i0 + ii < D && j0 + lane < n) dW[static_cast<int64_t>(i0 + ii) * n + j0 + lane] = tile[lane][ii];
+  block_add(s, out);
 }
 
 size_t align256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 
 struct SolveWs {
-  double* L;
-  double* B;
-  double* SW;
-  double* scal;  // [0] ||Y||^2, [1] ||dW||^2, [2] <W, S W>
+  int32_t Dp, np, kn;      // D to 128, d_out to 64 and to 32
+  int32_t t_d, t_n;        // 64-row tiles of the ops over D (one spare: a 128-row tile may start with the
+                           // last) and over d_out
+  uint8_t *op_a, *op_b;    // op_b (W) and the factor share their memory: X W is formed first
+  int64_t* fix;
+  double* B;               // by columns [d_out][Dp]: X W, then Y, then Z
+  uint8_t *op_panel, *op_s, *op_y, *op_i, *op_it;
+  double *inv, *inv_t;
+  int64_t* diag;
+  int32_t *t, *ea, *eb, *es, *ei, *eit;
+  double* scal;            // [0] ||Y||^2, [1] ||dW||^2, [2] tr(W^T S W)
   int* flag;
+  size_t bytes;
 };
 
 SolveWs carve(void* ws, int D, int d_out) {
-  uint8_t* p = static_cast<uint8_t*>(ws);
   SolveWs w;
-  w.L = reinterpret_cast<double*>(p);
-  p += align256(static_cast<size_t>(D) * D * 8);
-  w.B = reinterpret_cast<double*>(p);
-  p += align256(static_cast<size_t>(D) * d_out * 8);
-  w.SW = reinterpret_cast<double*>(p);
-  p += align256(static_cast<size_t>(D) * d_out * 8);
-  w.scal = reinterpret_cast<double*>(p);
-  p += 256;
-  w.flag = reinterpret_cast<int*>(p);
+  w.Dp = (D + TB - 1) / TB * TB;
+  w.np = (d_out + 63) / 64 * 64;
+  w.kn = (d_out + 31) / 32 * 32;
+  w.t_d = w.Dp / 64 + 1;
+  w.t_n = w.np / 64;
+  uint8_t* p = static_cast<uint8_t*>(ws);
+  auto take = [&](size_t bytes) {
+    uint8_t* r = p;
+    p += align256(bytes);
+    return r;
+  };
+  const size_t Dp = w.Dp, chunk_d = static_cast<size_t>(w.t_d) * SL_TILE, chunk_n = static_cast<size_t>(w.t_n) * SL_TILE;
+  const size_t ka = Dp > static_cast<size_t>(w.kn) ? Dp : w.kn;
+  w.op_a = take(ka / SL_K * chunk_d);
+  const size_t opb = Dp / SL_K * chunk_n, fix = Dp * Dp * 8;
+  w.op_b = take(opb > fix ? opb : fix);
+  w.fix = reinterpret_cast<int64_t*>(w.op_b);
+  w.B = reinterpret_cast<double*>(take(Dp * static_cast<size_t>(d_out) * 8));
+  w.op_panel = take(NB / SL_K * chunk_d);
+  w.op_s = take(TB / SL_K * chunk_n);
+  w.op_y = take(TB / SL_K * chunk_n);
+  w.op_i = take(TB / SL_K * chunk_d);
+  w.op_it = take(TB / SL_K * chunk_d);
+  w.inv = reinterpret_cast<double*>(take(Dp * TB * 8));
+  w.inv_t = reinterpret_cast<double*>(take(Dp * TB * 8));
+  w.diag = reinterpret_cast<int64_t*>(take(Dp * NB * 8));
+  w.t = reinterpret_cast<int32_t*>(take(Dp * 4));
+  w.ea = reinterpret_cast<int32_t*>(take((Dp / TB) * Dp * 4));
+  w.eb = reinterpret_cast<int32_t*>(take(static_cast<size_t>(w.np) * 4));
+  w.es = reinterpret_cast<int32_t*>(take(static_cast<size_t>(w.np) * 4));
+  w.ei = reinterpret_cast<int32_t*>(take(Dp * 4));
+  w.eit = reinterpret_cast<int32_t*>(take(Dp * 4));
+  w.scal = reinterpret_cast<double*>(take(256));
+  w.flag = reinterpret_cast<int*>(w.scal + 4);
+  w.bytes = static_cast<size_t>(p - static_cast<uint8_t*>(ws));
   return w;
 }
 
-cudaError_t gemm(int M, int N, int K, MatRef A, MatRef B, double* C, int64_t ldc, double alpha,
-                 double beta, bool lower_only, cudaStream_t s) {
-  if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-  dim3 grid((N + TB - 1) / TB, (M + TB - 1) / TB);
-  dgemm_kernel<<<grid, 256, 0, s>>>(M, N, K, A, B, C, ldc, alpha, beta, lower_only ? 1 : 0);
-  return cudaGetLastError();
+template <typename T>
+cudaError_t slice_rows(const T* src, int64_t ld, int rows, int ks, int seg_k, int n_seg, int64_t seg_src, int grid_rows,
+                       int n_t, int lower, uint8_t* op, int32_t* exps, int exp_ld, cudaStream_t s) {
+  const SliceParams p{src, ld, rows, ks, seg_k, seg_src, n_t, lower, exp_ld, op, exps};
+  return launch_pdl(slice_rows_kernel<T>, dim3(grid_rows / 8, n_seg), dim3(256), 0, s, p);
 }
 
-int grid_for(int64_t n, int threads) {
-  int64_t b = (n + threads - 1) / threads;
-  if (b > 152 * 16) b = 152 * 16;
-  return static_cast<int>(b < 1 ? 1 : b);
+template <typename T>
+cudaError_t slice_cols(const T* src, int64_t ld, int rows, int ks, int seg_k, int n_seg, int64_t seg_src, int grid_rows,
+                       int n_t, int lower, uint8_t* op, int32_t* exps, int exp_ld, cudaStream_t s) {
+  const SliceParams p{src, ld, rows, ks, seg_k, seg_src, n_t, lower, exp_ld, op, exps};
+  return launch_pdl(slice_cols_kernel<T>, dim3((grid_rows + 31) / 32, n_seg), dim3(seg_k > 512 ? 1024 : 256), 0, s, p);
 }
 
 }  // namespace
 
-size_t ls_solve_ws_bytes(int32_t D, int32_t d_out) {
-  return align256(static_cast<size_t>(D) * D * 8) + 2 * align256(static_cast<size_t>(D) * d_out * 8) + 512;
-}
+size_t ls_solve_ws_bytes(int32_t D, int32_t d_out) { return carve(nullptr, D, d_out).bytes; }
 
 ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d_out, double lambda,
                          float* dW, double* eps_out, void* ws, cudaStream_t s) {
-  SolveWs w = carve(ws, D, d_out);
+  const SolveWs w = carve(ws, D, d_out);
+  const int Dp = w.Dp, nb = Dp / TB;
   const int64_t ldg = 2 * static_cast<int64_t>(D);
-  const int64_t nDo = static_cast<int64_t>(D) * d_out;
+  const int64_t chunk_d = static_cast<int64_t>(w.t_d) * SL_TILE, chunk_n = static_cast<int64_t>(w.t_n) * SL_TILE;
+  int dev = 0, sms = 152;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
 #define ISPA_CK(x)                            \
   do {                                        \
     if ((x) != cudaSuccess) return ISPA_ERR_CUDA; \
   } while (0)
-  ISPA_CK(cudaMemsetAsync(w.scal, 0, 256 + sizeof(int), s));
-  form_spd_kernel<<<grid_for(static_cast<int64_t>(D) * D, 256), 256, 0, s>>>(gram, D, lambda, w.L);
-  ISPA_CK(cudaGetLastError());
-  // Cholesky, right-looking
-  for (int k0 = 0; k0 < D; k0 += NB) {
-    const int nb = D - k0 < NB ? D - k0 : NB;
-    potrf_diag_kernel<<<1, 256, 0, s>>>(w.L, D, k0, nb, w.flag);
-    ISPA_CK(cudaGetLastError());
-    const int rest = D - k0 - nb;
-    if (rest > 0) {
-      trsm_panel_kernel<<<(rest + 127) / 128, 128, 0, s>>>(w.L, D, k0, nb);
-      ISPA_CK(cudaGetLastError());
-      double* L22 = w.L + static_cast<int64_t>(k0 + nb) * D + (k0 + nb);
-      const double* L21 = w.L + static_cast<int64_t>(k0 + nb) * D + k0;
-      ISPA_CK(gemm(rest, rest, nb, MatRef{L21, D, M_F64}, MatRef{L21, D, M_F64_T}, L22, D, -1.0, 1.0,
-                   true, s));
-    }
+  SlGemm base{};
+  base.status = device_status_ptr();
+  if (!base.status) return ISPA_ERR_CUDA;
+  base.flag = w.flag;
+  base.wait_limit_ns = wait_limit_ns();
+  base.n_split = 1;
+  ISPA_CK(set_smem_limit_once(reinterpret_cast<const void*>(inverse_kernel), INV_SMEM));
+  ISPA_CK(set_smem_limit_once(reinterpret_cast<const void*>(panel_kernel), PANEL_SMEM));
+  ISPA_CK(cudaMemsetAsync(w.scal, 0, 256, s));
+  ISPA_CK(launch_pdl(equil_kernel, dim3((Dp + 255) / 256), dim3(256), 0, s, gram, D, Dp, lambda, w.t, w.flag));
+
+  // tr(W^T S W) = sum_ij S_ij (W W^T)_ij: W's rows sliced over d_out
+  ISPA_CK(slice_rows(W, d_out, D, d_out, w.kn, 1, 0, Dp, w.t_d, 0, w.op_a, w.ea, 0, s));
+  {
+    SlGemm p = base;
+    p.a = p.b = w.op_a;
+    p.a_chunk = p.b_chunk = chunk_d;
+    p.ea = p.eb = w.ea;
+    // the sum over the contraction index too can be cut: as many pieces of at least two flushes
+    // as make the last wave's idle SMs a small part of the whole
+    const int mt = Dp / 128, chunks = w.kn / SL_K;
+    p.n_split = chunks / (2 * SG_FLUSH) < 1 ? 1 : (chunks / (2 * SG_FLUSH) > 8 ? 8 : chunks / (2 * SG_FLUSH));
+    while (p.n_split > 1 && mt * (mt + 1) > 8 * sms) --p.n_split;
+    p.n_tiles = mt * (mt + 1) * p.n_split;
+    p.n_chunks = chunks;
+    p.row_end = D;
+    p.ld = ldg;
+    p.sym = gram + static_cast<int64_t>(D) * ldg + D;
+    p.dot = w.scal + 2;
+    ISPA_CK(launch_slice_gemm<SL_DOT>(p, sms, s));
   }
-  // B = X W
-  ISPA_CK(gemm(D, d_out, D, MatRef{gram + D, ldg, M_F32}, MatRef{W, d_out, M_F32}, w.B, d_out, 1.0, 0.0,
-               false, s));
-  // forward substitution
-  for (int k0 = 0; k0 < D; k0 += NB) {
-    const int nb = D - k0 < NB ? D - k0 : NB;
-    trsv_fwd_kernel<<<(d_out + 127) / 128, 128, 0, s>>>(w.L, D, k0, nb, w.B, d_out);
-    ISPA_CK(cudaGetLastError());
-    const int rest = D - k0 - nb;
-    if (rest > 0)
-      ISPA_CK(gemm(rest, d_out, nb, MatRef{w.L + static_cast<int64_t>(k0 + nb) * D + k0, D, M_F64},
-                   MatRef{w.B + static_cast<int64_t>(k0) * d_out, d_out, M_F64},
-                   w.B + static_cast<int64_t>(k0 + nb) * d_out, d_out, -1.0, 1.0, false, s));
+  // B = 2^-t X W
+  ISPA_CK(slice_rows(gram + D, ldg, D, D, Dp, 1, 0, Dp, w.t_d, 0, w.op_a, w.ea, 0, s));
+  ISPA_CK(slice_cols(W, d_out, d_out, D, Dp, 1, 0, w.np, w.t_n, 0, w.op_b, w.eb, 0, s));
+  {
+    SlGemm p = base;
+    p.a = w.op_a;
+    p.b = w.op_b;
+    p.a_chunk = chunk_d;
+    p.b_chunk = chunk_n;
+    p.ea = w.ea;
+    p.eb = w.eb;
+    p.n_mt = Dp / 128;
+    p.n_nt = w.np / 64;
+    p.n_tiles = p.n_mt * p.n_nt;
+    p.n_chunks = Dp / SL_K;
+    p.row_end = Dp;
+    p.col_end = d_out;
+    p.ld = Dp;
+    p.out = w.B;
+    p.row_exp = w.t;
+    ISPA_CK(launch_slice_gemm<SL_STORE>(p, sms, s));
   }
-  dot_kernel<double><<<grid_for(nDo, 256), 256, 0, s>>>(w.B, nullptr, nDo, w.scal + 0);
-  ISPA_CK(cudaGetLastError());
-  // back substitution
-  const int last = ((D - 1) / NB) * NB;
-  for (int k0 = last; k0 >= 0; k0 -= NB) {
-    const int nb = D - k0 < NB ? D - k0 : NB;
-    trsv_bwd_kernel<<<(d_out + 127) / 128, 128, 0, s>>>(w.L, D, k0, nb, w.B, d_out);
-    ISPA_CK(cudaGetLastError());
-    if (k0 > 0)
-      ISPA_CK(gemm(k0, d_out, nb, MatRef{w.L + static_cast<int64_t>(k0) * D, D, M_F64_T},
-                   MatRef{w.B + static_cast<int64_t>(k0) * d_out, d_out, M_F64}, w.B, d_out, -1.0, 1.0,
-                   false, s));
+  // Cholesky
+  ISPA_CK(launch_pdl(form_kernel, dim3(Dp, (Dp + 255) / 256), dim3(256), 0, s, gram, D, Dp, lambda,
+                     static_cast<const int32_t*>(w.t), w.fix, w.flag));
+  for (int k0 = 0; k0 < Dp; k0 += NB) {
+    const int rest = Dp - k0 - NB;
+    const PanelParams pp{w.fix, w.diag, Dp, k0, w.op_panel, w.t_d, w.ea, w.flag, base.status, base.wait_limit_ns};
+    ISPA_CK(launch_pdl(panel_kernel, dim3(rest > 0 ? rest / PR : 1), dim3(P_THREADS), PANEL_SMEM, s, pp));
+    if (rest <= 0) break;
+    SlGemm p = base;
+    p.a = p.b = w.op_panel;
+    p.a_chunk = p.b_chunk = chunk_d;
+    p.ea = p.eb = w.ea;
+    p.row0 = p.col0 = k0 + NB;
+    const int mt = (rest + 127) / 128;
+    p.n_tiles = mt * (mt + 1);
+    p.n_chunks = NB / SL_K;
+    p.row_end = Dp;
+    p.ld = Dp;
+    p.out = w.fix;
+    ISPA_CK(launch_slice_gemm<SL_CHOL>(p, sms, s));
   }
-  dot_kernel<double><<<grid_for(nDo, 256), 256, 0, s>>>(w.B, nullptr, nDo, w.scal + 1);
-  ISPA_CK(cudaGetLastError());
-  to_f32_kernel<<<grid_for(nDo, 256), 256, 0, s>>>(w.B, dW, nDo);
-  ISPA_CK(cudaGetLastError());
-  // <W, S W>
-  ISPA_CK(gemm(D, d_out, D, MatRef{gram + static_cast<int64_t>(D) * ldg + D, ldg, M_F32_SYM},
-               MatRef{W, d_out, M_F32}, w.SW, d_out, 1.0, 0.0, false, s));
-  dot_kernel<float><<<grid_for(nDo, 256), 256, 0, s>>>(w.SW, W, nDo, w.scal + 2);
-  ISPA_CK(cudaGetLastError());
-  double scal[3];
-  int flag = 0;
-  ISPA_CK(cudaMemcpyAsync(scal, w.scal, sizeof(scal), cudaMemcpyDeviceToHost, s));
-  ISPA_CK(cudaMemcpyAsync(&flag, w.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  ISPA_CK(launch_pdl(inverse_kernel, dim3(TB / IC, nb), dim3(256), INV_SMEM, s, static_cast<const int64_t*>(w.fix),
+                     static_cast<const int64_t*>(w.diag), Dp, w.inv, w.inv_t));
+  ISPA_CK(slice_rows(static_cast<const double*>(w.inv), TB, Dp, TB, TB, 1, 0, Dp, w.t_d, 0, w.op_i, w.ei, 0, s));
+  ISPA_CK(slice_rows(static_cast<const double*>(w.inv_t), TB, Dp, TB, TB, 1, 0, Dp, w.t_d, 0, w.op_it, w.eit, 0, s));
+
+  // One block step of a substitution: block row k of B becomes inv(L_kk) (or its transpose) times itself, and
+  // rows [r0, r1) lose their product with it.
+  auto step = [&](int k, const uint8_t* op_i, const int32_t* e_i, int r0, int r1) -> cudaError_t {
+    SlGemm p = base;
+    p.b = w.op_s;
+    p.a_chunk = chunk_d;
+    p.b_chunk = chunk_n;
+    p.eb = w.es;
+    p.n_nt = w.np / 64;
+    p.n_chunks = TB / SL_K;
+    p.col_end = d_out;
+    p.ld = Dp;
+    p.out = w.B;
+    cudaError_t e = slice_rows(static_cast<const double*>(w.B) + k * TB, Dp, d_out, TB, TB, 1, 0, w.np, w.t_n, 0, w.op_s,
+                               w.es, 0, s);
+    if (e != cudaSuccess) return e;
+    p.a = op_i;
+    p.ea = e_i;
+    p.row0 = k * TB;
+    p.row_end = k * TB + TB;
+    p.n_mt = 1;
+    p.n_tiles = p.n_nt;
+    if ((e = launch_slice_gemm<SL_STORE>(p, sms, s)) != cudaSuccess || r0 >= r1) return e;
+    if ((e = slice_rows(static_cast<const double*>(w.B) + k * TB, Dp, d_out, TB, TB, 1, 0, w.np, w.t_n, 0, w.op_y, w.es,
+                        0, s)) != cudaSuccess)
+      return e;
+    p.b = w.op_y;
+    p.a = w.op_a + static_cast<int64_t>(k) * (TB / SL_K) * chunk_d;
+    p.ea = w.ea + static_cast<int64_t>(k) * Dp;
+    p.row0 = r0;
+    p.row_end = r1;
+    p.n_mt = (r1 - r0) / 128;
+    p.n_tiles = p.n_mt * p.n_nt;
+    return launch_slice_gemm<SL_SUB>(p, sms, s);
+  };
+  // forward: the rows below block column k, sliced over its 128 columns
+  if (nb > 1)
+    ISPA_CK(slice_cols(static_cast<const int64_t*>(w.fix), Dp, Dp, TB, TB, nb - 1, static_cast<int64_t>(TB) * Dp, Dp,
+                       w.t_d, 1, w.op_a, w.ea, Dp, s));
+  for (int k = 0; k < nb; ++k) ISPA_CK(step(k, w.op_i, w.ei, (k + 1) * TB, Dp));
+  const int64_t nB = static_cast<int64_t>(Dp) * d_out;
+  const unsigned dot_grid = static_cast<unsigned>(nB / 2048 < 1 ? 1 : (nB / 2048 < 8 * sms ? nB / 2048 : 8 * sms));
+  ISPA_CK(launch_pdl(sumsq_kernel, dim3(dot_grid), dim3(256), 0, s, static_cast<const double*>(w.B), nB, w.scal));
+  // backward: the columns left of block row k, sliced over its 128 rows
+  if (nb > 1)
+    ISPA_CK(slice_rows(static_cast<const int64_t*>(w.fix), Dp, Dp, TB, TB, nb, TB, Dp, w.t_d, -1, w.op_a, w.ea, Dp, s));
+  for (int k = nb - 1; k >= 0; --k) ISPA_CK(step(k, w.op_it, w.eit, 0, k * TB));
+  ISPA_CK(launch_pdl(finish_kernel, dim3((D + 31) / 32, (d_out + 31) / 32), dim3(256), 0, s,
+                     static_cast<const double*>(w.B), D, Dp, d_out, static_cast<const int32_t*>(w.t), dW, w.scal + 1));
+  struct {
+    double scal[4];
+    int flag;
+  } h;
+  ISPA_CK(cudaMemcpyAsync(&h, w.scal, 4 * sizeof(double) + sizeof(int), cudaMemcpyDeviceToHost, s));
   ISPA_CK(cudaStreamSynchronize(s));
 #undef ISPA_CK
-  if (eps_out) *eps_out = scal[2] - scal[0] - lambda * scal[1];
-  return flag ? ISPA_ERR_NOT_SPD : ISPA_OK;
+  if (eps_out) *eps_out = h.scal[2] - h.scal[0] - lambda * h.scal[1];
+  if (h.flag & 2) return ISPA_ERR_TIMEOUT;
+  return h.flag ? ISPA_ERR_NOT_SPD : ISPA_OK;
 }
 
 }  // namespace ispa
