@@ -50,7 +50,13 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <map>
+#include <mutex>
+#include <tuple>
+
 #include "internal.h"
+#include "pdl.cuh"
 #include "ptx.cuh"
 
 namespace ispa {
@@ -92,7 +98,7 @@ struct Cfg {
   static constexpr int K_TILE = QK8 ? BN * HD : NBOX * KBOX;
   static constexpr int V_BOX8 = 128 * HD;                  // [HD rows][128 keys] e4m3 = 16 KB
   static constexpr int V_TILE = PV8 ? 2 * V_BOX8 : NBOX * KBOX;
-  static constexpr int PV_STEPS = PV8 ? BN / 32 : BN / 16;   // UMMAs of one P V
+  [[maybe_unused]] static constexpr int PV_STEPS = PV8 ? BN / 32 : BN / 16;   // UMMAs of one P V
   static constexpr float RESCALE = PV8 ? 4.0f : RESCALE_THRESHOLD;   // lazy rescale bound (log2)
   static constexpr float P_SHIFT = PV8 ? 4.0f : 0.0f;      // log2 of the scale P gets before rounding
   static constexpr int KST = (HD == 128 && !QK8) ? 2 : 4;  // K stages
@@ -180,6 +186,12 @@ __device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
   return r;
 }
 
+__device__ __forceinline__ int cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(r));
+  return static_cast<int>(r);
+}
+
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float r;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
@@ -188,6 +200,11 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 
 }  // namespace
 
+// SPLIT: the instance for items that leave SMs idle (see split_plan).  A cluster works on one item:
+// rank r of c visits the key tiles [n r / c, n (r + 1) / c), and at the end each CTA leaves its
+// unnormalised O, m and l in its shared memory (the stages are free by then) and merges 128 / c
+// rows over the cluster through distributed shared memory, the LSE fusion of Eq. 11-12.  No
+// workspace, no second launch, no dual mode.
 // TRACE: the instance launched while a trace buffer is set records the per-tile events of
 // ispa_debug_set_trace (first work item of CTA (0, 0)); the production instances contain no
 // trace code at all (even an untaken clock64 read constrains instruction scheduling: it cost 6 %
@@ -206,7 +223,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // epilogue's reads of O.
 // The TMA thread asks for the next item a few tiles before the end of the current one and
 // publishes it (or "none") to the UMMA thread and the softmax warps through a two-slot mailbox.
-template <int HD, bool QK8, bool PV8, bool TRACE>
+template <int HD, bool QK8, bool PV8, bool TRACE, bool SPLIT>
 __global__ void __launch_bounds__(NTHREADS, 1)
     attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_kr,
                 const __grid_constant__ CUtensorMap tm_vr, const __grid_constant__ CUtensorMap tm_kc,
@@ -287,7 +304,22 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
-  const int n_tiles = p.n_tiles;
+  // this CTA's first tile and tile count of an item (all of it unless SPLIT)
+  int tile0 = 0, n_tiles = p.n_tiles, item = p.item0 + static_cast<int>(blockIdx.x);
+  if constexpr (SPLIT) {
+    const int rank = static_cast<int>(cluster_ctarank()), c = cluster_size();
+    item = p.item0 + static_cast<int>(blockIdx.x) / c;
+    tile0 = p.n_tiles * rank / c;
+    n_tiles = p.n_tiles * (rank + 1) / c - tile0;
+  } else {
+    pdl_trigger();   // a split launch of the remaining items may take the SMs that run out of work
+  }
+  int seg0 = 0, off0 = 0;   // segment cursor of the first tile
+  if constexpr (SPLIT) {
+    int skip = tile0;
+    for (int n; skip >= (n = (p.seg[seg0].count + BN - 1) / BN); ++seg0) skip -= n;
+    off0 = skip * BN;
+  }
   // tile events of the CTA's first item (global tile index = item tile index there)
   auto tr = [&](int g, int ev) {
     if constexpr (TRACE) {
@@ -306,8 +338,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       const uint32_t sQ = sbase + C::OFF_Q;
       // item (q tile, head) of the K cursor, and the head of the item before it: V trails K by
       // at most one tile, so it is on one of the two
-      int kq = static_cast<int>(blockIdx.x), kh = static_cast<int>(blockIdx.y), prev_h = kh;
-      bool can_steal = true;     // no try_cancel has failed yet
+      int kq = item % p.n_qt, kh = item / p.n_qt, prev_h = kh;
+      bool can_steal = !SPLIT;   // no try_cancel has failed yet (a split item's cluster takes no other)
       int n_req = 0, n_resp = 0;  // try_cancel requests issued / responses consumed
       int nq = 0;                 // Q tiles issued
       auto request = [&]() {
@@ -324,8 +356,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       };
       // the request for the item after item k goes out this many K tiles before its end
       const int req_at = n_tiles > 4 ? n_tiles - 4 : 0;
-      int kk = 0, kj = 0, kseg = 0, koff = 0;   // K cursor: item, tile of the item, segment walk
-      int vk = 0, vj = 0, vseg = 0, voff = 0;   // V cursor
+      int kk = 0, kj = 0, kseg = seg0, koff = off0;   // K cursor: item, tile of the item, segment walk
+      int vk = 0, vj = 0, vseg = seg0, voff = off0;   // V cursor
       int t = 0, tv = 0;                        // global K and V tiles issued
       bool k_live = true, ok = true;
       load_q();
@@ -368,7 +400,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             load_q();
             if (req_at == 0) request();
           }
-          if (kj == p.drop_k_tile) break;   // debug: this load never goes out (timeout-path test)
+          if (tile0 + kj == p.drop_k_tile) break;   // debug: this load never goes out (timeout-path test)
           const int ks = t % C::KST;
           // K_t's stage held K_t-KST; S_t-2 complete means K_t-2 (and every older K) has been
           // read.  S_t cannot complete before K_t lands, so this barrier is never a phase ahead.
@@ -386,10 +418,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (n_req > n_resp) {
               if (!mbar_wait(b.clc, n_resp & 1, wc, 12, kk)) break;
               ++n_resp;
-              int cx, cy;
-              if (clc_query(clc_resp, cx, cy)) {
-                nx = cx;
-                ny = cy;
+              int cx;
+              if (clc_query(clc_resp, cx)) {
+                cx += p.item0;
+                nx = cx % p.n_qt;
+                ny = cx / p.n_qt;
               } else {
                 can_steal = false;
               }
@@ -588,7 +621,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int row = quarter * 32 + lane;
     const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     const int D = p.num_heads * HD;
-    int q_tile = blockIdx.x, head = blockIdx.y;   // the current item
+    int q_tile = item % p.n_qt, head = item / p.n_qt;   // the current item
     int qrow = 0;
     bool row_ok = false;
     float sl2_ring = p.scale_log2, sl2_chunk = p.scale_log2;
@@ -752,18 +785,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // log2-domain score scale; with 8-bit Q and K it also carries the per-head code scales,
       // which differ between ring keys and chunk keys
       if constexpr (QK8) {
-        const int n_qt = (p.n_q + BM - 1) / BM;
-        const float qs = p.q_scale[static_cast<int64_t>(head) * n_qt + q_tile];   // [H][query blocks]
+        const float qs = p.q_scale[static_cast<int64_t>(head) * p.n_qt + q_tile];   // [H][query blocks]
         sl2_ring = p.scale_log2 * qs * p.kr_scale[head];
         sl2_chunk = p.scale_log2 * qs * p.kc_scale[head];
       }
       m_run = -INFINITY;
       l_run = 0.f;
-      seg = off = 0;
+      seg = seg0;
+      off = off0;
       for (int j = 0; j < n_tiles; ++j) {
         const int g = base + j;
         const int sb = g & 1;
-        if (p.dual && j == p.n_local_tiles && j > 0) {
+        if (!SPLIT && p.dual && j == p.n_local_tiles && j > 0) {
           // A_loc snapshot: O and l hold exactly the local tiles 0..j-1.
           const float l_loc = row_l();
           if (ok) ok = wait_o(g - 1, 7);
@@ -871,6 +904,30 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const float l_row = row_l();   // overlaps the last P V
         if (ok) ok = wait_o(base + n_tiles - 1, 11);
         if (ok) tc_fence_after();
+        if constexpr (SPLIT) {
+          // This half of the row of O, unnormalised, into the stages (every load has landed and
+          // every UMMA has read them): 16-byte chunk q of row r at q ^ (r & 7).
+          if (ok) {
+            float4* xo = reinterpret_cast<float4*>(smem) + row * (HD / 4);
+#pragma unroll 1
+            for (int c = 0; c < C::O_HALF / 32; ++c) {
+              uint32_t r[32];
+              const int c0 = half * C::O_HALF + 32 * c;
+              tmem_ld32(trow + C::COL_O + c0, r);
+              tmem_wait_ld32(r);
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                xo[(c0 / 4 + q) ^ (row & 7)] =
+                    make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]),
+                                __uint_as_float(r[4 * q + 3]));
+            }
+          }
+          if (half == 0) {   // block 1 of the exchange area: m and l of the row
+            x_max[2 * BM + row] = m_run;
+            x_max[3 * BM + row] = ok ? l_row : 0.f;
+          }
+          break;
+        }
         if (p.dual && p.n_local_tiles >= n_tiles) emit(ok, l_row, p.out_loc, p.lse_loc, false);
         emit(ok, l_row, p.out, p.lse, p.dual != 0);
         if (threadIdx.x == 0 && k == 0) tr(0, 15);   // epilogue stored
@@ -892,6 +949,42 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (SPLIT) {
+    cluster_sync();   // every CTA's partial state is in its shared memory
+    if (warp < N_SOFT_WARPS) {
+      const int rank = static_cast<int>(cluster_ctarank()), c = cluster_size();
+      const int q_tile = item % p.n_qt, head = item / p.n_qt;
+      const float vs = PV8 ? p.v_scale[head] : 1.f;
+      // one warp per row, four columns per lane
+      for (int r = rank + c * warp; r < BM && q_tile * BM + r < p.n_q; r += c * N_SOFT_WARPS) {
+        const uint32_t xm = sbase + C::OFF_X + (2 * BM + r) * 4;
+        const uint32_t xo = sbase + (r * (HD / 4) + ((lane % (HD / 4)) ^ (r & 7))) * 16;
+        float m = -INFINITY;
+        for (int i = 0; i < c; ++i) m = fmaxf(m, cluster_ld1(cluster_map(xm, i)));
+        float l = 0.f;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int i = 0; i < c; ++i) {
+          // a CTA none of whose keys the row sees (frame-causal) has m = -inf and zeros
+          const float w = ex2_approx(cluster_ld1(cluster_map(xm, i)) - m);
+          l = fmaf(w, cluster_ld1(cluster_map(xm + BM * 4, i)), l);
+          const float4 v = cluster_ld4(cluster_map(xo, i));
+          o.x = fmaf(w, v.x, o.x);
+          o.y = fmaf(w, v.y, o.y);
+          o.z = fmaf(w, v.z, o.z);
+          o.w = fmaf(w, v.w, o.w);
+        }
+        const float inv = vs / l;
+        const size_t qrow = static_cast<size_t>(q_tile) * BM + r;
+        if (lane < HD / 4)
+          reinterpret_cast<uint2*>(p.out + (qrow * p.num_heads + head) * HD)[lane] =
+              make_uint2(pack_bf16x2(o.x * inv, o.y * inv), pack_bf16x2(o.z * inv, o.w * inv));
+        if (p.lse && lane == 0)
+          p.lse[static_cast<size_t>(head) * p.n_q + qrow] = (m - C::P_SHIFT + __log2f(l)) * 0.69314718055994531f;
+      }
+    }
+    cluster_sync();   // no CTA leaves while another still reads its shared memory
+    pdl_wait();       // the launch before this one (the other items) completes before this one does
+  }
   if (warp == WARP_MMA) {
     tc_fence_after();
     tmem_dealloc(tmem, TMEM_COLS);
@@ -899,21 +992,116 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
 }
 
+// Clusters of c CTAs of this kernel that the device holds at once (asked once per device and kernel).
+static int max_clusters(const void* func, int c, int smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int>, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(dev, func, c);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(c));
+  cfg.blockDim = dim3(NTHREADS);
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned>(c);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, func, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  known[key] = n;
+  return n;
+}
+
+// How many of the last items run as clusters, and of how many CTAs.  `items` whole items keep all SMs
+// busy but for the last, partial wave of r = items % sms: that wave (all of it when items < sms) is
+// split over c CTAs an item if that shortens it.  Measured (head_dim 128): a wave takes 8.3 us and
+// 1.06 us a key tile, a split wave 13 us and as much a tile of its longest CTA.  So in tiles a wave
+// costs n, a split one ceil(r / clusters at once) rounds of ceil(n / c) + 5, and 4 more for each round after
+// the first (its CTAs start over).  A gain below a tenth of the wave isn't taken, and after whole
+// items only a single round: at hidden 5120 a third of the last of ten waves saved on paper was 1 % lost.
+// One item an SM against split, start to end: 2 items of 80 tiles 94 -> 23 us, 38 of 40 tiles 52 -> 29,
+// 76 of 80 tiles 95 -> 59, 160 of 40 tiles 100 -> 70, 8 of 8 tiles 17.1 -> 16.5.
+struct SplitPlan {
+  int items, c;
+};
+template <typename F>
+static SplitPlan split_plan(int items, int n_tiles, int sms, F&& clusters) {
+  const int r = items % sms;
+  SplitPlan best{0, 1};
+  int cost = n_tiles - n_tiles / 10;
+  for (int c = 2; r > 0 && c <= 8 && 2 * c <= n_tiles; ++c) {
+    const int n = clusters(c);
+    if (n <= 0) continue;
+    const int rounds = (r + n - 1) / n;
+    if (rounds > 1 && items > sms) continue;
+    const int k = rounds * ((n_tiles + c - 1) / c + 5) + (rounds - 1) * 4;
+    if (k < cost) {
+      cost = k;
+      best = SplitPlan{r, c};
+    }
+  }
+  return best;
+}
+
 template <int HD, bool QK8, bool TRACE = false, bool PV8 = false>
 static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, const CUtensorMap* tvr,
-                             const CUtensorMap* tkc, const CUtensorMap* tvc, const AttnParams& p,
-                             cudaStream_t s) {
+                             const CUtensorMap* tkc, const CUtensorMap* tvc, AttnParams p, cudaStream_t s) {
   using C = Cfg<HD, QK8, PV8>;
-  int dev = 0;
+  const auto whole = attn_kernel<HD, QK8, PV8, TRACE, false>;
+  // Not with 8-bit P V: its probabilities are rounded to e4m3 against the running maximum, and a
+  // CTA's own maximum would round them otherwise (within the same bound, but 2.6 % of the output).
+  // Not in the dual pass: its discrepancy is a difference of outputs and would move with them.
+  const auto split = attn_kernel<HD, QK8, false, TRACE, true>;
+  int dev = 0, sms = 152;
   cudaGetDevice(&dev);
-  {
-    const cudaError_t e =
-        set_smem_limit_once(reinterpret_cast<const void*>(attn_kernel<HD, QK8, PV8, TRACE>), C::SMEM);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(whole), C::SMEM);
+  if (e != cudaSuccess) return e;
+  e = set_smem_limit_once(reinterpret_cast<const void*>(split), Cfg<HD, QK8, false>::SMEM);
+  if (e != cudaSuccess) return e;
+  p.n_qt = (p.n_q + BM - 1) / BM;
+  const int64_t all = static_cast<int64_t>(p.n_qt) * p.num_heads;
+  if (all > INT32_MAX) return cudaErrorInvalidValue;
+  const int items = static_cast<int>(all);
+  SplitPlan plan{0, 1};
+  if (!PV8 && !p.dual)
+    plan = split_plan(items, p.n_tiles, sms,
+                      [&](int c) { return max_clusters(reinterpret_cast<const void*>(split), c, C::SMEM); });
+  const int first = items - plan.items;
+  p.item0 = 0;
+  if (first > 0) {
+    whole<<<dim3(static_cast<unsigned>(first)), NTHREADS, C::SMEM, s>>>(*tq, *tkr, *tvr, *tkc, *tvc, p);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  dim3 grid((p.n_q + BM - 1) / BM, p.num_heads);
-  attn_kernel<HD, QK8, PV8, TRACE><<<grid, NTHREADS, C::SMEM, s>>>(*tq, *tkr, *tvr, *tkc, *tvc, p);
-  return cudaGetLastError();
+  if (plan.items > 0) {
+    p.item0 = first;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(plan.items * plan.c));
+    cfg.blockDim = dim3(NTHREADS);
+    cfg.dynamicSmemBytes = C::SMEM;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = static_cast<unsigned>(plan.c);
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // after the whole items' launch only: that one starts after everything before it has completed
+    cfg.numAttrs = first > 0 ? 2 : 1;
+    e = cudaLaunchKernelEx(&cfg, split, *tq, *tkr, *tvr, *tkc, *tvc, p);
+  }
+  return e;
 }
 
 cudaError_t launch_attention(int head_dim, const CUtensorMap* tq, const CUtensorMap* tkr,

@@ -31,6 +31,8 @@ struct AttnParams {
   int32_t num_heads;
   int32_t n_seg;           // segments in seg[]
   int32_t n_tiles;         // total key tiles over all segments
+  int32_t n_qt;            // query tiles; item i = (query tile i % n_qt, head i / n_qt)
+  int32_t item0;           // first item of the launch
   int32_t n_local_tiles;   // dual: tiles of the local set (they come first)
   int32_t dual;            // 1 = emit A_loc snapshot and discrepancy partials
   float scale_log2;        // softmax scale * log2(e)

@@ -165,24 +165,53 @@ __device__ __forceinline__ void clc_try_cancel(uint32_t resp_smem, uint32_t bar)
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
-// Decode a completed response: true and the cancelled CTA's (blockIdx.x, blockIdx.y) if a CTA
-// was cancelled, false if the request failed.
-__device__ __forceinline__ bool clc_query(uint32_t resp_smem, int& x, int& y) {
-  uint32_t ok, cx = 0, cy = 0;
+// Decode a completed response: true and the cancelled CTA's blockIdx.x if a CTA was cancelled,
+// false if the request failed.
+__device__ __forceinline__ bool clc_query(uint32_t resp_smem, int& x) {
+  uint32_t ok, cx = 0;
   asm volatile(
       "{\n\t.reg .b128 rr;\n\t.reg .pred p;\n\t.reg .b64 lo, hi;\n\t"
-      "ld.shared.v2.b64 {lo, hi}, [%3];\n\t"
+      "ld.shared.v2.b64 {lo, hi}, [%2];\n\t"
       "mov.b128 rr, {lo, hi};\n\t"
       "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, rr;\n\t"
       "selp.u32 %0, 1, 0, p;\n\t"
       "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, rr;\n\t"
-      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::y.b32.b128 %2, rr;\n\t}"
-      : "=r"(ok), "+r"(cx), "+r"(cy)
+      "}"
+      : "=r"(ok), "+r"(cx)
       : "r"(resp_smem)
       : "memory");
   x = static_cast<int>(cx);
-  y = static_cast<int>(cy);
   return ok != 0;
+}
+
+// ---------------------------------------------------------------- thread-block clusters
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// All threads of all CTAs of the cluster; shared-memory writes before it are visible to every CTA after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Address of the shared-memory location `addr` of this CTA in the CTA of rank `rank`.
+__device__ __forceinline__ uint32_t cluster_map(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 cluster_ld4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(addr)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float cluster_ld1(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
 }
 
 // ---------------------------------------------------------------- TMA
