@@ -98,7 +98,7 @@ struct Cfg {
   static constexpr int K_TILE = QK8 ? BN * HD : NBOX * KBOX;
   static constexpr int V_BOX8 = 128 * HD;                  // [HD rows][128 keys] e4m3 = 16 KB
   static constexpr int V_TILE = PV8 ? 2 * V_BOX8 : NBOX * KBOX;
-  [[maybe_unused]] static constexpr int PV_STEPS = PV8 ? BN / 32 : BN / 16;   // UMMAs of one P V
+  static constexpr int PV_STEPS = PV8 ? BN / 32 : BN / 16;   // UMMAs of one P V
   static constexpr float RESCALE = PV8 ? 4.0f : RESCALE_THRESHOLD;   // lazy rescale bound (log2)
   static constexpr float P_SHIFT = PV8 ? 4.0f : 0.0f;      // log2 of the scale P gets before rounding
   static constexpr int KST = (HD == 128 && !QK8) ? 2 : 4;  // K stages
@@ -311,9 +311,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     item = p.item0 + static_cast<int>(blockIdx.x) / c;
     tile0 = p.n_tiles * rank / c;
     n_tiles = p.n_tiles * (rank + 1) / c - tile0;
-  } else {
-    pdl_trigger();   // a split launch of the remaining items may take the SMs that run out of work
   }
+  // The kernel before this one may still run: nothing it writes (q, k, v, the ring, scales) has been
+  // touched so far.  A split launch after whole items is the exception (wait_first = 0): it starts only
+  // once those have passed this point, and waits for them at its end.
+  if (!SPLIT || p.wait_first) pdl_wait();
+  pdl_trigger();   // the next launch may take the SMs that run out of work
   int seg0 = 0, off0 = 0;   // segment cursor of the first tile
   if constexpr (SPLIT) {
     int skip = tile0;
@@ -983,7 +986,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       }
     }
     cluster_sync();   // no CTA leaves while another still reads its shared memory
-    pdl_wait();       // the launch before this one (the other items) completes before this one does
+    if (!p.wait_first) pdl_wait();   // the launch of the whole items completes before this one does
   }
   if (warp == WARP_MMA) {
     tc_fence_after();
@@ -1078,13 +1081,14 @@ static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, cons
                       [&](int c) { return max_clusters(reinterpret_cast<const void*>(split), c, C::SMEM); });
   const int first = items - plan.items;
   p.item0 = 0;
+  p.wait_first = 1;
   if (first > 0) {
-    whole<<<dim3(static_cast<unsigned>(first)), NTHREADS, C::SMEM, s>>>(*tq, *tkr, *tvr, *tkc, *tvc, p);
-    e = cudaGetLastError();
+    e = launch_pdl(whole, dim3(static_cast<unsigned>(first)), dim3(NTHREADS), C::SMEM, s, *tq, *tkr, *tvr, *tkc, *tvc, p);
     if (e != cudaSuccess) return e;
   }
   if (plan.items > 0) {
     p.item0 = first;
+    p.wait_first = first == 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(plan.items * plan.c));
     cfg.blockDim = dim3(NTHREADS);
@@ -1097,8 +1101,7 @@ static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, cons
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    // after the whole items' launch only: that one starts after everything before it has completed
-    cfg.numAttrs = first > 0 ? 2 : 1;
+    cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, split, *tq, *tkr, *tvr, *tkc, *tvc, p);
   }
   return e;

@@ -33,6 +33,7 @@ struct AttnParams {
   int32_t n_tiles;         // total key tiles over all segments
   int32_t n_qt;            // query tiles; item i = (query tile i % n_qt, head i / n_qt)
   int32_t item0;           // first item of the launch
+  int32_t wait_first;      // 1: wait for the kernel before this launch; 0 (split items after whole ones): at the end
   int32_t n_local_tiles;   // dual: tiles of the local set (they come first)
   int32_t dual;            // 1 = emit A_loc snapshot and discrepancy partials
   float scale_log2;        // softmax scale * log2(e)

@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "pdl.cuh"
 #include "ptx.cuh"
 
 namespace ispa {
@@ -49,6 +50,8 @@ constexpr int CACHE = 12;
 __global__ void __launch_bounds__(256) quant_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows,
                                                          int cols, uint8_t* __restrict__ q,
                                                          float* __restrict__ scale) {
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int nw = cols / 8;   // 16-byte words of bf16 per row
   const int64_t warps = static_cast<int64_t>(gridDim.x) * (blockDim.x >> 5);
@@ -234,6 +237,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_wait();   // the codes and scales may come from the kernel before this one
+  pdl_trigger();
   const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
 
   if (warp == 0) {
@@ -383,8 +388,7 @@ cudaError_t launch_gemm_bn(const uint8_t* a_q, const float* a_scale, const uint8
   int dev_sms = 152;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = p.n_tiles < dev_sms ? p.n_tiles : dev_sms;
-  w8a8_gemm_kernel<BN><<<grid, Q_THREADS, C::SMEM, s>>>(ta, tw, p);
-  return cudaGetLastError();
+  return launch_pdl(w8a8_gemm_kernel<BN>, dim3(grid), dim3(Q_THREADS), C::SMEM, s, ta, tw, p);
 }
 
 }  // namespace
@@ -395,9 +399,8 @@ cudaError_t launch_quant_rows(const void* x, int64_t rows, int32_t cols, uint8_t
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int64_t want = (rows + 7) / 8;   // one warp per row, 8 warps per block
   const int64_t blocks = want < static_cast<int64_t>(sms) * 16 ? want : static_cast<int64_t>(sms) * 16;
-  quant_rows_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(static_cast<const __nv_bfloat16*>(x), rows, cols,
-                                                                    q, scale);
-  return cudaGetLastError();
+  return launch_pdl(quant_rows_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s,
+                    static_cast<const __nv_bfloat16*>(x), rows, static_cast<int>(cols), q, scale);
 }
 
 cudaError_t launch_quant_weight(const float* W, const float* dW, int32_t D, int32_t Dout, uint8_t* q_t, float* scale,
