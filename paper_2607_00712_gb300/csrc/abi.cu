@@ -837,7 +837,7 @@ ispa_status ispa_kv_append_qk8(ispa_kv_ring* ring, const void* k_new, const void
   for (int i = 0; i < n_frames; ++i) slots[i] = slot_of(ring, ring->frames_written + i);
   const int64_t ring_tok = static_cast<int64_t>(ring->capacity_frames) * ring->tokens_per_frame;
   if (launch_append_qk8(slots, n_frames, ring->tokens_per_frame, ring->num_heads, ring->head_dim, ring_tok, k_new,
-                        v_new, ring->k, ring->v, k_scale, stream) != cudaSuccess)
+                        v_new, ring->k, ring->v, k_scale, nullptr, 0, stream) != cudaSuccess)
     return ISPA_ERR_CUDA;
   ring->frames_written += n_frames;
   return ISPA_OK;
@@ -848,7 +848,7 @@ ispa_status ispa_quantize_vt_e4m3(const void* x, int64_t n, int32_t H, int32_t d
   if (!x || !scale || !qt || n <= 0 || H <= 0 || !aligned16(x) || !aligned16(qt) || ld < n || ld % 16 != 0)
     return ISPA_ERR_INVALID_ARG;
   if (d != 128) return ISPA_ERR_UNSUPPORTED;
-  if (launch_quant_vt(x, n, H, d, scale, qt, ld, 0, 0, nullptr, stream) != cudaSuccess) return ISPA_ERR_CUDA;
+  if (launch_quant_vt(x, n, H, scale, qt, ld, stream) != cudaSuccess) return ISPA_ERR_CUDA;
   return ISPA_OK;
 }
 
@@ -865,11 +865,8 @@ ispa_status ispa_kv_append_kv8(ispa_kv_ring* ring, const void* k_new, const void
   for (int i = 0; i < n_frames; ++i) slots[i] = slot_of(ring, ring->frames_written + i);
   const int32_t P = ring->tokens_per_frame;
   const int64_t ring_tok = static_cast<int64_t>(ring->capacity_frames) * P;
-  if (launch_append_qk8(slots, n_frames, P, ring->num_heads, ring->head_dim, ring_tok, k_new, v_new, ring->k,
-                        nullptr, k_scale, stream) != cudaSuccess ||
-      launch_quant_vt(v_new, static_cast<int64_t>(n_frames) * P, ring->num_heads, ring->head_dim, v_scale,
-                      static_cast<uint8_t*>(ring->v), ispa_ring_vt_stride(ring), P, n_frames, slots,
-                      stream) != cudaSuccess)
+  if (launch_append_qk8(slots, n_frames, P, ring->num_heads, ring->head_dim, ring_tok, k_new, v_new, ring->k, ring->v,
+                        k_scale, v_scale, ispa_ring_vt_stride(ring), stream) != cudaSuccess)
     return ISPA_ERR_CUDA;
   ring->frames_written += n_frames;
   return ISPA_OK;

@@ -122,13 +122,14 @@ cudaError_t launch_quant_q_blocks(const void* x, int64_t n, int32_t H, int32_t d
                                   cudaStream_t s);
 cudaError_t launch_quant_given(const void* x, int64_t n, int32_t H, int32_t d, const float* scale, uint8_t* q,
                                cudaStream_t s);
-// d-major e4m3 values: out[h][c][key] (key = t, or slots[t / P] * P + t % P when n_frames > 0);
-// d = 128, ld % 16 == 0, P % 4 == 0.
-cudaError_t launch_quant_vt(const void* x, int64_t n, int32_t H, int32_t d, const float* scale, uint8_t* out,
-                            int64_t ld, int32_t P, int32_t n_frames, const int32_t* slots, cudaStream_t s);
+// d-major e4m3 values: out[h][c][t], d = 128, ld % 16 == 0.
+cudaError_t launch_quant_vt(const void* x, int64_t n, int32_t H, const float* scale, uint8_t* out, int64_t ld,
+                            cudaStream_t s);
+// vt_scale: null (values copied as bf16), or the values' per-head scales: v_dst then takes d-major codes
+// of row stride vt_ld in the frames' slots (d = 128, P % 4 == 0).
 cudaError_t launch_append_qk8(const int32_t* slots, int32_t n_frames, int32_t P, int32_t H, int32_t d,
                               int64_t ring_tok, const void* k_src, const void* v_src, void* k_dst, void* v_dst,
-                              const float* k_scale, cudaStream_t s);
+                              const float* k_scale, const float* vt_scale, int64_t vt_ld, cudaStream_t s);
 
 // ------------------------------------------------------------ misc
 int* device_status_ptr();  // library status word in the current context (nullptr on error)
