@@ -115,94 +115,132 @@ __device__ __forceinline__ void store_digits8(const int64_t* xi, uint8_t* dst) {
   }
 }
 
+// What a slice kernel takes: grid.y segments z of `rows` rows x `ks` k.  Segments either follow each other
+// along k (L's block columns: z_k chunks apart in the op, exponents per segment) or are blocks down a
+// diagonal (z_rows rows apart, in the same chunks).
 struct SliceParams {
   const void* src;
   int64_t ld;          // elements between rows (k-contiguous source) or between k (row-contiguous source)
-  int32_t rows, ks;    // valid rows and k of the source (of one segment)
-  int32_t seg_k;       // k of a segment, a multiple of 32 (the padded k when there is one segment)
-  int64_t seg_src;     // elements between the segments' first values in the source
+  int64_t z_src;       // elements between the segments' first values
+  int32_t rows, ks;    // valid rows and k of a segment
+  int32_t rows_total, ks_total;   // if not 0: segment z has at most rows_total - z z_rows rows (those past
+                                  // them are not written), ks_total - z (z_k or z_rows) k
+  int32_t k_pad;       // k written: a multiple of 32, zeros past the valid ones (z_k segments: only those)
+  int32_t z_rows;      // op rows between segments
+  int32_t z_k;         // k between segments in the op: 0 or k_pad
+  int32_t z_exp;       // exponents between segments
+  int32_t win;         // z_k segments: if not 0, only the rows of the segment's own window of so many rows, and
+                       // a window's segments start again at the op's first chunk
+  int32_t lower;       // z_k segments: 1: only the rows past the segment's k, -1: only those before them
   int32_t n_t;         // tiles of 64 rows of the op
-  int32_t lower;       // 1: segment z needs the rows above z * seg_k + seg_k - 1 only; -1: the rows below z * seg_k
-  int32_t exp_ld;      // exponents of segment z start at exps + z * exp_ld
   uint8_t* op;
   int32_t* exps;
 };
+__device__ __forceinline__ int sl_rows(const SliceParams& p, int z) {
+  return p.rows_total ? min(p.rows, p.rows_total - z * p.z_rows) : p.rows;
+}
+__device__ __forceinline__ int sl_ks(const SliceParams& p, int z) {
+  return p.ks_total ? min(p.ks, p.ks_total - z * (p.z_k ? p.z_k : p.z_rows)) : p.ks;
+}
+__device__ __forceinline__ int sl_z(const SliceParams& p, int z) { return p.win ? z % (p.win / p.z_k) : z; }
+__device__ __forceinline__ int sl_row0(const SliceParams& p, int z) { return p.win ? z * p.z_k / p.win * p.win : 0; }
+__device__ __forceinline__ int sl_pad(const SliceParams& p, int ks) {
+  return p.z_k ? (ks + SL_K - 1) / SL_K * SL_K : p.k_pad;
+}
+// Which of a segment's values are there (the others are taken as zero): all, k <= row, or k >= row.
+enum SlTri : int { SL_FULL, SL_LOWER, SL_UPPER };
+template <int TRI>
+__device__ __forceinline__ bool sl_there(int row, int k) {
+  return TRI == SL_FULL || (TRI == SL_LOWER ? k <= row : k >= row);
+}
 
-// Source with k contiguous.  One CTA per 8 rows (blockIdx.x) and segment (blockIdx.y): warp w finds row
-// w's exponent, then the warps take the segment's chunks in turn, a thread 8 k of one row, a
-// warp 8 rows x 32 k, so that each slice of it is one contiguous 512-byte store.
-template <typename T>
-__global__ void __launch_bounds__(256) slice_rows_kernel(const SliceParams p) {
+// Source with k contiguous.  One CTA (8 warps, 16 for long rows) per 8 rows (blockIdx.x) and segment
+// (blockIdx.y): first a warp or two find a row's exponent, then the warps take the segment's chunks in turn, a
+// thread 8 k of one row, a warp 8 rows x 32 k, so that each slice of it is one contiguous 512-byte
+// store.  (Loading once, in the second pass's order, and reducing over the CTA is slower, 10.1 us
+// against 9.1 on average in a 5120 x 5120 solve: each of those loads touches 32 sectors.)
+template <typename T, int TRI>
+__global__ void __launch_bounds__(512) slice_rows_kernel(const SliceParams p) {
   using S = SliceSrc<T>;
   pdl_wait();
   pdl_trigger();
-  __shared__ int e_sh[8];
-  const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = blockIdx.x * 8;
-  if (p.lower > 0 && r0 < (z + 1) * p.seg_k) return;
-  if (p.lower < 0 && r0 >= z * p.seg_k) return;
-  const T* src = static_cast<const T*>(p.src) + z * p.seg_src;
+  __shared__ typename S::Mag red[2][8];
+  const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
+  const int zc = sl_z(p, z), r0 = sl_row0(p, z) + blockIdx.x * 8;
+  if (p.lower > 0 && r0 < (z + 1) * p.k_pad) return;
+  if (p.lower < 0 && r0 >= z * p.k_pad) return;
+  const int rows = sl_rows(p, z), ks = sl_ks(p, z), k_pad = sl_pad(p, ks);
+  if (p.rows_total && r0 >= rows) return;
+  const T* src = static_cast<const T*>(p.src) + z * p.z_src + r0 * p.ld;
   typename S::Mag m = 0;
-  if (r0 + warp < p.rows) {
-    const T* row = src + (r0 + warp) * p.ld;
-    for (int k = lane; k < p.ks; k += 32) m = max(m, S::mag(row[k]));
-  }
+  {
+    const int r = warp & 7;
+    const T* row = src + r * p.ld;
+    if (r0 + r < rows) {
+      for (int k = lane + 32 * (warp >> 3); k < ks; k += 4 * n_warp)
+        if (sl_there<TRI>(r0 + r, k)) m = max(m, S::mag(row[k]));
+    }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if (lane == 0) {
-    const int e = S::exp_of(m);
-    e_sh[warp] = e;
-    p.exps[z * p.exp_ld + r0 + warp] = e;
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) red[warp >> 3][r] = m;
   }
   __syncthreads();
   const int r = lane & 7, kc = lane >> 3;
-  const int E = e_sh[r];
-  const bool live = r0 + r < p.rows && E != SL_NAN;
-  const T* row = src + (r0 + r) * p.ld;
-  for (int c = warp; c < p.seg_k / SL_K; c += 8) {
+  m = n_warp > 8 ? max(red[0][r], red[1][r]) : red[0][r];
+  const int E = S::exp_of(m);
+  if (threadIdx.x < 8) p.exps[zc * p.z_exp + z * p.z_rows + r0 + r] = E;
+  const bool live = r0 + r < rows && E != SL_NAN;
+  const T* row = src + r * p.ld;
+  for (int c = warp; c < k_pad / SL_K; c += n_warp) {
     int64_t xi[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = c * SL_K + kc * 8 + i;
-      xi[i] = live && k < p.ks ? S::fixed(row[k], E) : 0;
+      xi[i] = live && k < ks && sl_there<TRI>(r0 + r, k) ? S::fixed(row[k], E) : 0;
     }
-    const int64_t ch = static_cast<int64_t>(z) * (p.seg_k / SL_K) + c;
-    store_digits8(xi, p.op + sl_offset(ch, p.n_t, r0 + r, kc));
+    store_digits8(xi, p.op + sl_offset(zc * (p.z_k / SL_K) + c, p.n_t, z * p.z_rows + r0 + r, kc));
   }
 }
 
-// Source with rows contiguous (k strided).  One CTA (8 warps, 32 for long segments) per 32 rows and segment; lane = row, so
-// every load is a contiguous run of the source and every slice store four 128-byte runs.
-template <typename T>
+// Source with rows contiguous (k strided).  One CTA (8 warps, 32 for long segments) per 32 rows and
+// segment; lane = row, so every load is a contiguous run of the source and every slice store four
+// 128-byte runs.  Where that leaves SMs idle the stores are split over blockIdx.z, each CTA finding the exponents
+// for itself: 57 -> 21 us for a 1536 x 1536 W.
+template <typename T, int TRI>
 __global__ void __launch_bounds__(1024) slice_cols_kernel(const SliceParams p) {
   using S = SliceSrc<T>;
   pdl_wait();
   pdl_trigger();
   __shared__ typename S::Mag red[32][32];
   const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
-  const int r0 = blockIdx.x * 32, r = r0 + lane;
-  if (p.lower > 0 && r0 < (z + 1) * p.seg_k) return;
-  if (p.lower < 0 && r0 >= z * p.seg_k) return;
-  const T* src = static_cast<const T*>(p.src) + z * p.seg_src + r;
-  const bool in = r < p.rows;
+  const int zc = sl_z(p, z), r0 = sl_row0(p, z) + blockIdx.x * 32, r = r0 + lane;
+  if (p.lower > 0 && r0 < (z + 1) * p.k_pad) return;
+  if (p.lower < 0 && r0 >= z * p.k_pad) return;
+  const int rows = sl_rows(p, z), ks = sl_ks(p, z), k_pad = sl_pad(p, ks);
+  if (p.rows_total && r0 >= rows) return;
+  const T* src = static_cast<const T*>(p.src) + z * p.z_src + r;
+  const bool in = r < rows;
   typename S::Mag m = 0;
   if (in) {
 #pragma unroll 8
-    for (int k = warp; k < p.ks; k += n_warp) m = max(m, S::mag(src[k * p.ld]));
+    for (int k = warp; k < ks; k += n_warp)
+      if (sl_there<TRI>(r, k)) m = max(m, S::mag(src[k * p.ld]));
   }
   red[warp][lane] = m;
   __syncthreads();
   for (int w = 0; w < n_warp; ++w) m = max(m, red[w][lane]);
   const int E = S::exp_of(m);
-  if (r >= p.n_t * 64) return;
-  if (warp == 0) p.exps[z * p.exp_ld + r] = E;
+  if (z * p.z_rows + r >= p.n_t * 64) return;
+  if (warp == 0 && blockIdx.z == 0) p.exps[zc * p.z_exp + z * p.z_rows + r] = E;
   const bool live = in && E != SL_NAN;
-  for (int q = warp; q < p.seg_k / 8; q += n_warp) {
+  for (int q = warp + n_warp * blockIdx.z; q < k_pad / 8; q += n_warp * gridDim.z) {
     int64_t xi[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) xi[i] = live && 8 * q + i < p.ks ? S::fixed(src[(8 * q + i) * p.ld], E) : 0;
-    const int64_t ch = static_cast<int64_t>(z) * (p.seg_k / SL_K) + (q >> 2);
-    store_digits8(xi, p.op + sl_offset(ch, p.n_t, r, q & 3));
+    for (int i = 0; i < 8; ++i) {
+      const int k = 8 * q + i;
+      xi[i] = live && k < ks && sl_there<TRI>(r, k) ? S::fixed(src[k * p.ld], E) : 0;
+    }
+    store_digits8(xi, p.op + sl_offset(zc * (p.z_k / SL_K) + (q >> 2), p.n_t, z * p.z_rows + r, q & 3));
   }
 }
 

@@ -14,8 +14,8 @@
 // products with the inverses of L's 128 x 128 diagonal blocks, and tr(W^T S W) = sum_ij S_ij (W W^T)_ij, half
 // the work of S W and nothing to store.  Plain fp64 code ran all of it at 1.09 TFLOP/s, the chip's
 // fp64 rate: 782 ms at hidden 5120 and 33 ms at 1536 (where the panels' launches and latency counted
-// too), against 30.5 and 3.1 ms.  What bounds it now: at 5120 the products' tensor time and read-back (24
-// of 30 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
+// too), against 28.4 and 3.06 ms.  What bounds it now: at 5120 the products' tensor time and read-back (22
+// of 28 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
 // dW's error against 64-bit arithmetic (before its rounding to fp32) is 0.4 to 0.8 times the plain code's.
 //
 // The factorisation runs in fixed point.  Row and column i are scaled by a power of two (exactly)
@@ -39,6 +39,14 @@ namespace {
 
 constexpr int NB = 64;     // panel of the factorisation
 constexpr int TB = 128;    // block of the substitutions
+// Window of a large problem's substitutions.  Each block of 128 rows updates only the rows of its own
+// window at once; the others get one product with K = 512 for the window's four blocks, a quarter of the
+// read-modify-writes of B and of the pipeline fills: 30.7 -> 28.5 ms at 5120 x 5120 (the
+// updates alone 10.3 -> 8.1).  It costs two launches a window and small products that fill few SMs, so it starts
+// where the average update has 512 tiles: 3072 x 3072 (576 tiles) 10.11 -> 9.91 ms, 4096 x 4096 18.5 -> 17.65;
+// at 400 tiles (2560 x 2560) 7.28 -> 7.29, at 144 (1536 x 1536) 3.13 -> 3.19.
+constexpr int SB = 512;
+constexpr size_t SB_TILES = 512;
 constexpr int PR = 32;     // panel rows per CTA
 constexpr int FLAG_NOT_SPD = 1;
 
@@ -333,13 +341,15 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
   }
 }
 
-// Inverse of L's 128 x 128 diagonal blocks, fp64: inv[b][i][j] and its transpose.  One CTA per 8
-// columns of a block; thread (column, row group): right-looking substitution with its rows in registers.
+// Inverse I of L's 128 x 128 diagonal blocks, fp64.  The factor is stored by columns and leaves the other half of
+// its array free: I_ij goes to [i][j], where column i has no L (the 64 x 64 blocks on the diagonal are
+// L's in `diag`).  One CTA per 8 columns of a block; thread (column, row group): right-looking substitution with its
+// rows in registers.
 constexpr int IC = 8;
 constexpr int IG = 256 / IC;   // row groups
 constexpr int INV_SMEM = (TB * (TB + 1) + 2 * IC + TB) * 8;
-__global__ void __launch_bounds__(256) inverse_kernel(const int64_t* __restrict__ fix, const int64_t* __restrict__ diag,
-                                                      int Dp, double* __restrict__ inv, double* __restrict__ inv_t) {
+__global__ void __launch_bounds__(256) inverse_kernel(const int64_t* fix, const int64_t* __restrict__ diag,
+                                                      int Dp, double* inv) {
   extern __shared__ double sm[];
   double* l = sm;                        // by columns, [c][TB + 1]
   double* xs = sm + TB * (TB + 1);       // the current row of the solution, twice
@@ -377,13 +387,10 @@ __global__ void __launch_bounds__(256) inverse_kernel(const int64_t* __restrict_
     for (int m = k / IG; m < TB / IG; ++m)
       if (g + IG * m > k) x[m] = fma(-l[k * (TB + 1) + g + IG * m], v, x[m]);
   }
-  const int64_t base = static_cast<int64_t>(b) * TB * TB;
 #pragma unroll
   for (int m = 0; m < TB / IG; ++m) {
     const int i = g + IG * m, j = c0 + col;
-    const double v = i >= j ? x[m] : 0.0;
-    inv[base + i * TB + j] = v;
-    inv_t[base + j * TB + i] = v;
+    if (i >= j) inv[static_cast<int64_t>(b * TB + i) * Dp + b * TB + j] = x[m];
   }
 }
 
@@ -435,15 +442,15 @@ size_t align256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 
 struct SolveWs {
   int32_t Dp, np, kn;      // D to 128, d_out to 64 and to 32
+  int32_t win;             // rows of a window of the substitutions
   int32_t t_d, t_n;        // 64-row tiles of the ops over D (one spare: a 128-row tile may start with the
                            // last) and over d_out
   uint8_t *op_a, *op_b;    // op_b (W) and the factor share their memory: X W is formed first
   int64_t* fix;
   double* B;               // by columns [d_out][Dp]: X W, then Y, then Z
-  uint8_t *op_panel, *op_s, *op_y, *op_i, *op_it;
-  double *inv, *inv_t;
+  uint8_t *op_panel, *op_s, *op_n, *op_i, *op_it;
   int64_t* diag;
-  int32_t *t, *ea, *eb, *es, *ei, *eit;
+  int32_t *t, *ea, *en, *eb, *es, *ei, *eit;
   double* scal;            // [0] ||Y||^2, [1] ||dW||^2, [2] tr(W^T S W)
   int* flag;
   size_t bytes;
@@ -470,15 +477,16 @@ SolveWs carve(void* ws, int D, int d_out) {
   w.fix = reinterpret_cast<int64_t*>(w.op_b);
   w.B = reinterpret_cast<double*>(take(Dp * static_cast<size_t>(d_out) * 8));
   w.op_panel = take(NB / SL_K * chunk_d);
-  w.op_s = take(TB / SL_K * chunk_n);
-  w.op_y = take(TB / SL_K * chunk_n);
+  w.win = w.Dp > SB && Dp / 256 * static_cast<size_t>(w.t_n) >= SB_TILES ? SB : w.Dp;
+  const bool one = w.win == w.Dp;
+  w.op_s = take((one ? TB : SB) / SL_K * chunk_n);
+  w.op_n = one ? w.op_a : take(SB / SL_K * chunk_d);
   w.op_i = take(TB / SL_K * chunk_d);
   w.op_it = take(TB / SL_K * chunk_d);
-  w.inv = reinterpret_cast<double*>(take(Dp * TB * 8));
-  w.inv_t = reinterpret_cast<double*>(take(Dp * TB * 8));
   w.diag = reinterpret_cast<int64_t*>(take(Dp * NB * 8));
   w.t = reinterpret_cast<int32_t*>(take(Dp * 4));
-  w.ea = reinterpret_cast<int32_t*>(take((Dp / TB) * Dp * 4));
+  w.ea = reinterpret_cast<int32_t*>(take((Dp + w.win - 1) / w.win * Dp * 4));
+  w.en = reinterpret_cast<int32_t*>(take(w.win / TB * Dp * 4));
   w.eb = reinterpret_cast<int32_t*>(take(static_cast<size_t>(w.np) * 4));
   w.es = reinterpret_cast<int32_t*>(take(static_cast<size_t>(w.np) * 4));
   w.ei = reinterpret_cast<int32_t*>(take(Dp * 4));
@@ -489,18 +497,34 @@ SolveWs carve(void* ws, int D, int d_out) {
   return w;
 }
 
-template <typename T>
-cudaError_t slice_rows(const T* src, int64_t ld, int rows, int ks, int seg_k, int n_seg, int64_t seg_src, int grid_rows,
-                       int n_t, int lower, uint8_t* op, int32_t* exps, int exp_ld, cudaStream_t s) {
-  const SliceParams p{src, ld, rows, ks, seg_k, seg_src, n_t, lower, exp_ld, op, exps};
-  return launch_pdl(slice_rows_kernel<T>, dim3(grid_rows / 8, n_seg), dim3(256), 0, s, p);
+// One segment: rows x ks values, k padded to k_pad with zeros.
+SliceParams slice(const void* src, int64_t ld, int rows, int ks, int k_pad, int n_t, uint8_t* op, int32_t* exps) {
+  SliceParams p{};
+  p.src = src;
+  p.ld = ld;
+  p.rows = rows;
+  p.ks = ks;
+  p.k_pad = k_pad;
+  p.n_t = n_t;
+  p.op = op;
+  p.exps = exps;
+  return p;
 }
 
-template <typename T>
-cudaError_t slice_cols(const T* src, int64_t ld, int rows, int ks, int seg_k, int n_seg, int64_t seg_src, int grid_rows,
-                       int n_t, int lower, uint8_t* op, int32_t* exps, int exp_ld, cudaStream_t s) {
-  const SliceParams p{src, ld, rows, ks, seg_k, seg_src, n_t, lower, exp_ld, op, exps};
-  return launch_pdl(slice_cols_kernel<T>, dim3((grid_rows + 31) / 32, n_seg), dim3(seg_k > 512 ? 1024 : 256), 0, s, p);
+// grid_rows: rows of a segment in the op (multiples of 8, those past the valid ones are zeroed).
+template <typename T, int TRI = SL_FULL>
+cudaError_t slice_rows(const SliceParams& p, int grid_rows, int n_seg, cudaStream_t s) {
+  const dim3 grid(grid_rows / 8, n_seg);
+  return launch_pdl(slice_rows_kernel<T, TRI>, grid, dim3(p.k_pad > 512 ? 512 : 256), 0, s, p);
+}
+
+template <typename T, int TRI = SL_FULL>
+cudaError_t slice_cols(const SliceParams& p, int grid_rows, int n_seg, cudaStream_t s) {
+  dim3 grid((grid_rows + 31) / 32, n_seg);
+  const int warps = p.k_pad > 128 ? 32 : 8, most = p.k_pad / 8 / warps;   // parts with work for every warp
+  const int fill = 304 / static_cast<int>(grid.x * grid.y);
+  grid.z = fill < 1 || most < 1 ? 1 : (fill < most ? fill : most);
+  return launch_pdl(slice_cols_kernel<T, TRI>, grid, dim3(32 * warps), 0, s, p);
 }
 
 }  // namespace
@@ -532,7 +556,7 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
   ISPA_CK(launch_pdl(equil_kernel, dim3((Dp + 255) / 256), dim3(256), 0, s, gram, D, Dp, lambda, w.t, w.flag));
 
   // tr(W^T S W) = sum_ij S_ij (W W^T)_ij: W's rows sliced over d_out
-  ISPA_CK(slice_rows(W, d_out, D, d_out, w.kn, 1, 0, Dp, w.t_d, 0, w.op_a, w.ea, 0, s));
+  ISPA_CK(slice_rows<float>(slice(W, d_out, D, d_out, w.kn, w.t_d, w.op_a, w.ea), Dp, 1, s));
   {
     SlGemm p = base;
     p.a = p.b = w.op_a;
@@ -552,8 +576,8 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     ISPA_CK(launch_slice_gemm<SL_DOT>(p, sms, s));
   }
   // B = 2^-t X W
-  ISPA_CK(slice_rows(gram + D, ldg, D, D, Dp, 1, 0, Dp, w.t_d, 0, w.op_a, w.ea, 0, s));
-  ISPA_CK(slice_cols(W, d_out, d_out, D, Dp, 1, 0, w.np, w.t_n, 0, w.op_b, w.eb, 0, s));
+  ISPA_CK(slice_rows<float>(slice(gram + D, ldg, D, D, Dp, w.t_d, w.op_a, w.ea), Dp, 1, s));
+  ISPA_CK(slice_cols<float>(slice(W, d_out, d_out, D, Dp, w.t_n, w.op_b, w.eb), w.np, 1, s));
   {
     SlGemm p = base;
     p.a = w.op_a;
@@ -594,58 +618,95 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     p.out = w.fix;
     ISPA_CK(launch_slice_gemm<SL_CHOL>(p, sms, s));
   }
+  double* inv = reinterpret_cast<double*>(w.fix);
   ISPA_CK(launch_pdl(inverse_kernel, dim3(TB / IC, nb), dim3(256), INV_SMEM, s, static_cast<const int64_t*>(w.fix),
-                     static_cast<const int64_t*>(w.diag), Dp, w.inv, w.inv_t));
-  ISPA_CK(slice_rows(static_cast<const double*>(w.inv), TB, Dp, TB, TB, 1, 0, Dp, w.t_d, 0, w.op_i, w.ei, 0, s));
-  ISPA_CK(slice_rows(static_cast<const double*>(w.inv_t), TB, Dp, TB, TB, 1, 0, Dp, w.t_d, 0, w.op_it, w.eit, 0, s));
+                     static_cast<const int64_t*>(w.diag), Dp, inv));
+  const int64_t ld = Dp;
+  {
+    // I for the forward steps (rows i), I^T for the backward ones (rows j)
+    SliceParams q = slice(inv, ld, TB, TB, TB, w.t_d, w.op_i, w.ei);
+    q.z_src = TB * (ld + 1);
+    q.z_rows = TB;
+    ISPA_CK((slice_rows<double, SL_LOWER>(q, TB, nb, s)));
+    q.op = w.op_it;
+    q.exps = w.eit;
+    ISPA_CK((slice_cols<double, SL_UPPER>(q, TB, nb, s)));
+  }
 
-  // One block step of a substitution: block row k of B becomes inv(L_kk) (or its transpose) times itself, and
-  // rows [r0, r1) lose their product with it.
-  auto step = [&](int k, const uint8_t* op_i, const int32_t* e_i, int r0, int r1) -> cudaError_t {
-    SlGemm p = base;
-    p.b = w.op_s;
-    p.a_chunk = chunk_d;
-    p.b_chunk = chunk_n;
-    p.eb = w.es;
-    p.n_nt = w.np / 64;
-    p.n_chunks = TB / SL_K;
-    p.col_end = d_out;
-    p.ld = Dp;
-    p.out = w.B;
-    cudaError_t e = slice_rows(static_cast<const double*>(w.B) + k * TB, Dp, d_out, TB, TB, 1, 0, w.np, w.t_n, 0, w.op_s,
-                               w.es, 0, s);
-    if (e != cudaSuccess) return e;
-    p.a = op_i;
-    p.ea = e_i;
-    p.row0 = k * TB;
-    p.row_end = k * TB + TB;
-    p.n_mt = 1;
-    p.n_tiles = p.n_nt;
-    if ((e = launch_slice_gemm<SL_STORE>(p, sms, s)) != cudaSuccess || r0 >= r1) return e;
-    if ((e = slice_rows(static_cast<const double*>(w.B) + k * TB, Dp, d_out, TB, TB, 1, 0, w.np, w.t_n, 0, w.op_y, w.es,
-                        0, s)) != cudaSuccess)
-      return e;
-    p.b = w.op_y;
-    p.a = w.op_a + static_cast<int64_t>(k) * (TB / SL_K) * chunk_d;
-    p.ea = w.ea + static_cast<int64_t>(k) * Dp;
+  // B's rows [r0, r0 + n) sliced, over all columns
+  auto slice_b = [&](int r0, int n) {
+    return slice_rows<double>(slice(w.B + r0, Dp, d_out, n, n, w.t_n, w.op_s, w.es), w.np, 1, s);
+  };
+  SlGemm sub = base;
+  sub.b = w.op_s;
+  sub.a_chunk = chunk_d;
+  sub.b_chunk = chunk_n;
+  sub.eb = w.es;
+  sub.n_nt = w.np / 64;
+  sub.col_end = d_out;
+  sub.ld = Dp;
+  sub.out = w.B;
+  auto rows = [](SlGemm p, const uint8_t* op, const int32_t* exps, int r0, int r1, int k) {
+    p.a = op;
+    p.ea = exps;
     p.row0 = r0;
     p.row_end = r1;
     p.n_mt = (r1 - r0) / 128;
     p.n_tiles = p.n_mt * p.n_nt;
-    return launch_slice_gemm<SL_SUB>(p, sms, s);
+    p.n_chunks = k / SL_K;
+    return p;
   };
-  // forward: the rows below block column k, sliced over its 128 columns
-  if (nb > 1)
-    ISPA_CK(slice_cols(static_cast<const int64_t*>(w.fix), Dp, Dp, TB, TB, nb - 1, static_cast<int64_t>(TB) * Dp, Dp,
-                       w.t_d, 1, w.op_a, w.ea, Dp, s));
-  for (int k = 0; k < nb; ++k) ISPA_CK(step(k, w.op_i, w.ei, (k + 1) * TB, Dp));
+  // One block step of a substitution: block row k of B becomes inv(L_kk) (or its transpose) times itself, and
+  // rows [r0, r1) of its window lose their product with it.
+  auto step = [&](int k, const uint8_t* op_i, const int32_t* e_i, int r0, int r1) -> cudaError_t {
+    cudaError_t e = slice_b(k * TB, TB);
+    if (e == cudaSuccess) e = launch_slice_gemm<SL_STORE>(rows(sub, op_i, e_i, k * TB, (k + 1) * TB, TB), sms, s);
+    if (e != cudaSuccess || r0 >= r1) return e;
+    if ((e = slice_b(k * TB, TB)) != cudaSuccess) return e;
+    const int zc = k % (w.win / TB);
+    return launch_slice_gemm<SL_SUB>(rows(sub, w.op_n + static_cast<int64_t>(zc) * (TB / SL_K) * chunk_d,
+                                          w.en + static_cast<int64_t>(zc) * Dp, r0, r1, TB), sms, s);
+  };
+  // Rows [r0, r1) outside of window z lose their product with all of it.
+  auto far = [&](int z, int r0, int r1) -> cudaError_t {
+    const int n = Dp - z * w.win < w.win ? Dp - z * w.win : w.win;
+    const cudaError_t e = slice_b(z * w.win, n);
+    if (e != cudaSuccess) return e;
+    return launch_slice_gemm<SL_SUB>(rows(sub, w.op_a + static_cast<int64_t>(z) * (w.win / SL_K) * chunk_d,
+                                          w.ea + static_cast<int64_t>(z) * Dp, r0, r1, n), sms, s);
+  };
+  // L's values for both: blocks of 128 columns (forward; rows: backward) within the windows, the window's width outside
+  const int n_win = (Dp + w.win - 1) / w.win;
+  SliceParams near_l = slice(w.fix, ld, Dp, TB, TB, w.t_d, w.op_n, w.en), far_l = slice(w.fix, ld, Dp, w.win, w.win, w.t_d, w.op_a, w.ea);
+  near_l.rows_total = far_l.ks_total = Dp;
+  near_l.z_k = TB;
+  near_l.win = far_l.z_k = w.win;
+  near_l.z_exp = far_l.z_exp = Dp;
+  // forward
+  near_l.lower = far_l.lower = 1;
+  near_l.z_src = TB * ld;
+  far_l.z_src = w.win * ld;
+  if (nb > 1) ISPA_CK(slice_cols<int64_t>(near_l, w.win, nb, s));
+  if (n_win > 1) ISPA_CK(slice_cols<int64_t>(far_l, Dp, n_win - 1, s));
+  for (int z = 0; z < n_win; ++z) {
+    const int k1 = (z + 1) * (w.win / TB) < nb ? (z + 1) * (w.win / TB) : nb;
+    for (int k = z * (w.win / TB); k < k1; ++k) ISPA_CK(step(k, w.op_i, w.ei, (k + 1) * TB, k1 * TB));
+    if (k1 < nb) ISPA_CK(far(z, k1 * TB, Dp));
+  }
   const int64_t nB = static_cast<int64_t>(Dp) * d_out;
   const unsigned dot_grid = static_cast<unsigned>(nB / 2048 < 1 ? 1 : (nB / 2048 < 8 * sms ? nB / 2048 : 8 * sms));
   ISPA_CK(launch_pdl(sumsq_kernel, dim3(dot_grid), dim3(256), 0, s, static_cast<const double*>(w.B), nB, w.scal));
-  // backward: the columns left of block row k, sliced over its 128 rows
-  if (nb > 1)
-    ISPA_CK(slice_rows(static_cast<const int64_t*>(w.fix), Dp, Dp, TB, TB, nb, TB, Dp, w.t_d, -1, w.op_a, w.ea, Dp, s));
-  for (int k = nb - 1; k >= 0; --k) ISPA_CK(step(k, w.op_it, w.eit, 0, k * TB));
+  // backward
+  near_l.lower = far_l.lower = -1;
+  near_l.z_src = TB;
+  far_l.z_src = w.win;
+  if (nb > 1) ISPA_CK(slice_rows<int64_t>(near_l, w.win, nb, s));
+  if (n_win > 1) ISPA_CK(slice_rows<int64_t>(far_l, Dp, n_win, s));
+  for (int z = n_win - 1; z >= 0; --z) {
+    const int k1 = (z + 1) * (w.win / TB) < nb ? (z + 1) * (w.win / TB) : nb;
+    for (int k = k1 - 1; k >= z * (w.win / TB); --k) ISPA_CK(step(k, w.op_it, w.eit, z * w.win, k * TB));
+    if (z > 0) ISPA_CK(far(z, 0, z * w.win));
+  }
   ISPA_CK(launch_pdl(finish_kernel, dim3((D + 31) / 32, (d_out + 31) / 32), dim3(256), 0, s,
                      static_cast<const double*>(w.B), D, Dp, d_out, static_cast<const int32_t*>(w.t), dW, w.scal + 1));
   struct {

@@ -100,3 +100,9 @@ def test_a_nan_weight_stays_in_its_column():
     assert np.isnan(dW[:, 5]).all() and np.isnan(eps)
     keep = np.arange(n) != 5
     assert np.array_equal(dW[:, keep], clean[:, keep])
+
+
+@pytest.mark.parametrize("D,n,spread", [(520, 16384, 0.0), (700, 10900, 1.0), (1030, 6600, 0.0)])
+def test_solve_in_windows(D, n, spread):
+    # many columns: the substitutions go by windows of 512 rows, the last of which is partial
+    test_solve_matches_the_oracle(D, n, spread)
