@@ -144,13 +144,16 @@ bool encode_tmap_4d(CUtensorMap* m, const void* base, const uint64_t dims4[4], c
                     const uint32_t box4[4], bool u8 = false);   // u8: uint8 elements instead of bf16
 bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1,
                     uint64_t stride1_bytes, uint32_t b0, uint32_t b1);
-// uint8 elements, 128-byte swizzle, rank 2.
+// the same with 64-byte swizzle
+bool encode_tmap_2d_sw64(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1,
+                         uint64_t stride1_bytes, uint32_t b0, uint32_t b1);
 // fp32 [d1][d0] with 128-byte swizzle (the Gram state, for bulk reduce-adds)
 bool encode_tmap_2d_f32(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t stride1_bytes,
                         uint32_t b0, uint32_t b1);
 // uint8 (d0 inner, d1, d2) with 128-byte swizzle
 bool encode_tmap_3d_u8(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2,
                        uint64_t stride1_bytes, uint64_t stride2_bytes, uint32_t b0, uint32_t b1, uint32_t b2);
+// uint8 elements, 128-byte swizzle, rank 2
 bool encode_tmap_2d_u8(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t stride1_bytes,
                        uint32_t b0, uint32_t b1);
 uint64_t wait_limit_ns();

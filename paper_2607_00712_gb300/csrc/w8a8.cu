@@ -12,14 +12,18 @@
 // oracle's): amax = max |x|; inv = 448 / amax, scale = amax / 448 (both 1 for an all-zero
 // group); code = e4m3(x * inv), round to nearest even with saturation at +-448.
 //
-// GEMM: persistent, one CTA per SM looping over 128 x BN output tiles (BN = 256, 192 or 128,
-// whichever gives the shortest estimated run: waves of tiles x their cost); both operands
+// GEMM: persistent, one CTA per SM looping over 128 x BN output tiles (BN = 256, 192 or 128), or one pair of
+// CTAs over 256 x 256 tiles (cta_group::2), whichever gives the shortest estimated run; both operands
 // K-major with 128-byte swizzle (one 128-byte row = 128 codes = four K=32 UMMA steps), a
-// 4-stage TMA ring that runs on across tile boundaries, two accumulator sets in TMEM so that
+// 4-stage TMA ring (6 in a pair) that runs on across tile boundaries, two accumulator sets in TMEM so that
 // the epilogue of one tile (both scales, bf16 store) overlaps the UMMAs of the next; with
 // 128-column tiles each set has two accumulation chains that the k-steps alternate between.
-// Warp 0 issues TMA, warp 1 allocates TMEM and issues UMMAs, warps 2-5 drain TMEM (warp w
-// reads lanes 32 (w % 4) .. +31).  Every wait is bounded.
+// Warp 0 issues TMA, warp 1 allocates TMEM and issues UMMAs, warps 2-9 drain TMEM (warp w
+// reads lanes 32 (w % 4) .. +31 and half of the columns), give the set back at once, and store
+// through 32 x 32 blocks in shared memory and TMA.  (Stores from registers, a lane a row, were 32 cache lines an
+// instruction: 64 KB of a tile took 2 us that nothing hid after a CTA's last tile and that slowed the others.)
+// 4680 x 1536 -> 1536: 15.0 -> 11.5 us, -> 4608: 32.7 -> 24.8 us; 4680 x 5120 -> 5120: 79.6 -> 68.0 us (3.6
+// PFLOP/s).  Every wait is bounded.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -159,10 +163,12 @@ __global__ void col_scale_kernel(float* __restrict__ s, int Dout) {
 // ------------------------------------------------------------ GEMM
 constexpr int QM = 128;        // output rows (tokens) per tile
 constexpr int QK = 128;        // K (bytes = codes) per stage: one 128-byte swizzled row
-constexpr int Q_THREADS = 192;
+constexpr int Q_EPI = 8;         // read-back warps: two per TMEM lane quarter, half of the columns each
+constexpr int Q_BLOCK = 32 * 64;
+constexpr int Q_THREADS = 64 + 32 * Q_EPI;
 constexpr uint64_t Q_DRAIN_NS = 200ull * 1000 * 1000;
 
-template <int BN>
+template <int BN, bool PAIR>
 struct QCfg {
   // Persistent: one CTA per SM loops over output tiles.  Two accumulator sets in TMEM let the
   // epilogue of one tile overlap the UMMAs of the next; with 128-column tiles each set holds
@@ -170,36 +176,38 @@ struct QCfg {
   static_assert(BN == 128 || BN == 192 || BN == 256, "tile width");
   static constexpr int CHAINS = BN == 128 ? 2 : 1;
   static constexpr int SET = CHAINS * BN;         // TMEM columns per accumulator set
-  static constexpr int QST = 4;
+  static constexpr int QST = PAIR ? 6 : 4;
+  static constexpr int CTAS = PAIR ? 2 : 1;
+  static constexpr int BR = BN / CTAS;            // this CTA's rows of B
   static constexpr int A_BYTES = QM * QK;         // 16 KB
-  static constexpr int B_BYTES = BN * QK;         // 32, 24 or 16 KB
+  static constexpr int B_BYTES = BR * QK;         // 32, 24 or 16 KB, half of that in a pair
   static constexpr int STAGE = A_BYTES + B_BYTES;
-  static constexpr int OFF_BAR = QST * STAGE;
+  static constexpr int OFF_OUT = QST * STAGE;     // two blocks of 32 x 32 bf16 per read-back warp
+  static constexpr int OFF_BAR = OFF_OUT + Q_EPI * 2 * Q_BLOCK;
   static constexpr int N_BAR = 2 * QST + 4 + 1;   // full/empty per stage, set full/empty x2, drain
   static constexpr int SMEM = OFF_BAR + N_BAR * 8 + 16;
   // more than half of an SM's shared memory: one CTA per SM, so the 512-column TMEM
   // allocation never waits for another CTA
   static_assert(SMEM > 116 * 1024 && SMEM <= 232448 && STAGE % 1024 == 0, "shared memory layout");
-  static constexpr uint32_t IDESC = idesc_e4m3(QM, BN);
+  static constexpr uint32_t IDESC = idesc_e4m3(QM * CTAS, BN);
   static constexpr uint32_t TMEM_COLS = 512;      // the allocation (a power of two)
   static_assert(2 * SET <= 512, "two accumulator sets fit in TMEM");
 };
 
 struct GemmParams {
   int32_t T, D, Dout, n_kb;
-  int32_t n_mt, n_tiles;   // row tiles; all tiles (tile t: rows (t % n_mt), columns (t / n_mt))
+  int32_t n_mt, n_tiles;   // row tiles (of 256 rows for pairs); all tiles (tile t: rows (t % n_mt), columns (t / n_mt))
   const float* a_scale;
   const float* w_scale;
-  __nv_bfloat16* out;
   int* status;
   uint64_t wait_limit_ns;
 };
 
-template <int BN>
+template <int BN, bool PAIR>
 __global__ void __launch_bounds__(Q_THREADS, 1)
     w8a8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
-                     const GemmParams p) {
-  using C = QCfg<BN>;
+                     const __grid_constant__ CUtensorMap tm_out, const GemmParams p) {
+  using C = QCfg<BN, PAIR>;
   constexpr int QST = C::QST;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw;
@@ -215,6 +223,11 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
                  acce0 = accf0 + 16, drain_bar = acce0 + 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_kb = p.n_kb;
+  const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
+  const int unit = blockIdx.x / C::CTAS, units = gridDim.x / C::CTAS;   // one CTA or pair per output tile
+  // A pair's rank 0 issues the UMMAs: its full barriers count both CTAs' bytes, its set-empty barriers both
+  // CTAs' epilogue warps.  The stage-empty, set-full and drain barriers are each CTA's own,
+  // arrived at by commits that go to both.
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < QST; ++i) {
@@ -223,53 +236,76 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(accf0 + 8 * i, 1);
-      mbar_init(acce0 + 8 * i, 128);
+      mbar_init(acce0 + 8 * i, Q_EPI * C::CTAS);
     }
     mbar_init(drain_bar, 1);
     *abort_flag = 0;
     fence_mbar_init();
   }
+  if constexpr (PAIR) cluster_sync();   // both CTAs run and their barriers exist
   if (warp == 1) {
-    tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
-    tmem_relinquish();
+    if constexpr (PAIR) {
+      tmem_alloc_pair(smem_u32(tmem_slot), C::TMEM_COLS);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   pdl_wait();   // the codes and scales may come from the kernel before this one
   pdl_trigger();
   const WaitCtx wc{abort_flag, p.status, p.wait_limit_ns};
+  auto commit = [](uint32_t bar) {
+    if constexpr (PAIR) tc_commit_pair(bar);
+    else tc_commit(bar);
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       int g = 0;   // k-blocks issued over all tiles of this CTA
       bool ok = true;
-      for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x) {
-        const int m0 = (t % p.n_mt) * QM, n0 = (t / p.n_mt) * BN;
+      for (int t = unit; ok && t < p.n_tiles; t += units) {
+        const int m0 = ((t % p.n_mt) * C::CTAS + rank) * QM, n0 = (t / p.n_mt) * BN;
         for (int kb = 0; kb < n_kb; ++kb, ++g) {
           const int st = g % QST;
           if (!mbar_wait(empty0 + 8 * st, ((g / QST) & 1) ^ 1, wc, 31, g)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(full0 + 8 * st, C::STAGE);
+          if (rank == 0) mbar_arrive_expect_tx(full0 + 8 * st, C::CTAS * C::STAGE);
           const uint32_t sa = sbase + st * C::STAGE;
-          tma_load_2d(sa, &tm_a, full0 + 8 * st, kb * QK, m0);
-          tma_load_2d(sa + C::A_BYTES, &tm_w, full0 + 8 * st, kb * QK, n0);
+          if constexpr (PAIR) {
+            const uint32_t bar = cluster_map(full0 + 8 * st, 0);
+            tma_load_2d_pair(sa, &tm_a, bar, kb * QK, m0);
+            tma_load_2d_pair(sa + C::A_BYTES, &tm_w, bar, kb * QK, n0 + rank * C::BR);
+          } else {
+            tma_load_2d(sa, &tm_a, full0 + 8 * st, kb * QK, m0);
+            tma_load_2d(sa + C::A_BYTES, &tm_w, full0 + 8 * st, kb * QK, n0);
+          }
         }
       }
-      for (int i = g > QST ? g - QST : 0; i < g; ++i)
-        mbar_wait_drain(full0 + 8 * (i % QST), (i / QST) & 1, Q_DRAIN_NS);
+      if (rank == 0) {
+        for (int i = g > QST ? g - QST : 0; i < g; ++i)
+          mbar_wait_drain(full0 + 8 * (i % QST), (i / QST) & 1, Q_DRAIN_NS);
+      } else if (!ok) {
+        // after a timeout: rank 1's loads count on rank 0's barriers, so give those in flight time to land
+        const uint64_t t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 1000 * 1000) __nanosleep(1000);
+      }
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------ UMMA issuer
-    if (lane == 0) {
+    if (lane == 0 && rank == 0) {
       int g = 0, i = 0;
       bool ok = true;
-      for (int t = blockIdx.x; ok && t < p.n_tiles; t += gridDim.x, ++i) {
+      for (int t = unit; ok && t < p.n_tiles; t += units, ++i) {
         const int set = i & 1;
         // the epilogue has drained this set's previous tile (tile i - 2)
         if (!mbar_wait(acce0 + 8 * set, ((i >> 1) & 1) ^ 1, wc, 34, i)) break;
@@ -285,110 +321,128 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
           const uint32_t sa = sbase + st * C::STAGE, sb = sa + C::A_BYTES;
           // four K=32 steps inside the 128-byte swizzle row (alternating chains for BN 128)
 #pragma unroll
-          for (int k = 0; k < QK / 32; ++k)
-            umma_f8(acc + (C::CHAINS == 2 ? (k & 1) * BN : 0), sw128_desc(sa + 32 * k, 16, 1024),
-                    sw128_desc(sb + 32 * k, 16, 1024), C::IDESC, (kb > 0 || k >= C::CHAINS) ? 1u : 0u);
-          tc_commit(empty0 + 8 * st);
+          for (int k = 0; k < QK / 32; ++k) {
+            const uint32_t d = acc + (C::CHAINS == 2 ? (k & 1) * BN : 0), more = (kb > 0 || k >= C::CHAINS) ? 1u : 0u;
+            const uint64_t da = sw128_desc(sa + 32 * k, 16, 1024), db = sw128_desc(sb + 32 * k, 16, 1024);
+            if constexpr (PAIR) umma_f8_pair(d, da, db, C::IDESC, more);
+            else umma_f8(d, da, db, C::IDESC, more);
+          }
+          commit(empty0 + 8 * st);
         }
         if (!ok) break;
-        tc_commit(accf0 + 8 * set);
+        commit(accf0 + 8 * set);
       }
-      tc_commit(drain_bar);
-      mbar_wait_drain(drain_bar, 0, Q_DRAIN_NS);
+      commit(drain_bar);
     }
+    if (lane == 0) mbar_wait_drain(drain_bar, 0, rank == 0 ? Q_DRAIN_NS : p.wait_limit_ns + 2 * Q_DRAIN_NS);
     __syncwarp();
   } else {
-    // ------------------------------------------------------------ epilogue (warps 2-5)
-    const int quarter = warp & 3;
+    // ------------------------------------------------------------ epilogue (warps 2-9)
+    constexpr int HC = BN / 64;   // 32-column chunks of this warp's half
+    const int quarter = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* block = smem + C::OFF_OUT + (warp - 2) * 2 * Q_BLOCK;
     int i = 0;
-    for (int t = blockIdx.x; t < p.n_tiles; t += gridDim.x, ++i) {
+    for (int t = unit; t < p.n_tiles; t += units, ++i) {
       const int set = i & 1;
+      const int m0 = ((t % p.n_mt) * C::CTAS + rank) * QM, n0 = (t / p.n_mt) * BN + half * (BN / 2);
+      const int row = m0 + quarter * 32 + lane;
+      // the scales are here before the sums are
+      const float sa = row < p.T ? p.a_scale[row] : 0.f;
+      float sw[HC];   // of column 32 c + lane
+#pragma unroll
+      for (int c = 0; c < HC; ++c) sw[c] = p.w_scale[n0 + 32 * c + lane];
       if (!__all_sync(0xffffffffu, mbar_wait(accf0 + 8 * set, (i >> 1) & 1, wc, 33, i))) break;
       tc_fence_after();
-      const int m0 = (t % p.n_mt) * QM, n0 = (t / p.n_mt) * BN;
-      const int row = m0 + quarter * 32 + lane;
-      const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + set * C::SET;
-      const float sa = row < p.T ? p.a_scale[row] : 0.f;
-      __nv_bfloat16* orow = p.out + static_cast<size_t>(row) * p.Dout + n0;
-#pragma unroll 1
-      for (int c = 0; c < BN / 32; ++c) {
-        // the 32 columns' weight scales (the same for every lane), loaded before the TMEM wait
-        float sw[32];
-        const float4* sw4 = reinterpret_cast<const float4*>(p.w_scale + n0 + 32 * c);
+      const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + set * C::SET + half * (BN / 2);
+      // all loads out together, then the set goes back at once
+      uint32_t v[C::CHAINS * HC][32];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float4 t = sw4[q];
-          sw[4 * q] = t.x;
-          sw[4 * q + 1] = t.y;
-          sw[4 * q + 2] = t.z;
-          sw[4 * q + 3] = t.w;
-        }
-        uint32_t v0[32], v1[32];
-        tmem_ld32(taddr + 32 * c, v0);
-        tmem_wait_ld32(v0);
-        if constexpr (C::CHAINS == 2) {
-          tmem_ld32(taddr + BN + 32 * c, v1);
-          tmem_wait_ld32(v1);
-        }
-        if (row < p.T) {
-          uint32_t pk[16];
+      for (int c = 0; c < HC; ++c) {
+        tmem_ld32(taddr + 32 * c, v[c]);
+        if constexpr (C::CHAINS == 2) tmem_ld32(taddr + BN + 32 * c, v[HC + c]);
+      }
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            float s0 = __uint_as_float(v0[2 * e]), s1 = __uint_as_float(v0[2 * e + 1]);
+      for (int c = 0; c < C::CHAINS * HC; ++c) tmem_wait_ld32(v[c]);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if constexpr (PAIR) mbar_arrive_cluster(cluster_map(acce0 + 8 * set, 0));
+        else mbar_arrive(acce0 + 8 * set);
+      }
+      if (m0 + quarter * 32 >= p.T) continue;   // uniform over the warp; rows past T inside the block are clipped
+#pragma unroll
+      for (int c = 0; c < HC; ++c) {
+        uint8_t* b = block + (c & 1) * Q_BLOCK;
+        if (lane == 0) bulk_wait_read<1>();   // the store before last has read this block
+        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float s0 = __uint_as_float(v[c][8 * q + 2 * e]), s1 = __uint_as_float(v[c][8 * q + 2 * e + 1]);
             if constexpr (C::CHAINS == 2) {
-              s0 += __uint_as_float(v1[2 * e]);
-              s1 += __uint_as_float(v1[2 * e + 1]);
+              s0 += __uint_as_float(v[HC + c][8 * q + 2 * e]);
+              s1 += __uint_as_float(v[HC + c][8 * q + 2 * e + 1]);
             }
-            pk[e] = pack_bf16x2(__fmul_rn(__fmul_rn(s0, sa), sw[2 * e]), __fmul_rn(__fmul_rn(s1, sa), sw[2 * e + 1]));
+            pk[e] = pack_bf16x2(__fmul_rn(__fmul_rn(s0, sa), __shfl_sync(0xffffffffu, sw[c], 8 * q + 2 * e)),
+                                __fmul_rn(__fmul_rn(s1, sa), __shfl_sync(0xffffffffu, sw[c], 8 * q + 2 * e + 1)));
           }
-          uint4* d4 = reinterpret_cast<uint4*>(orow + 32 * c);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) d4[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+          // 64-byte swizzle: 16-byte word q of row r at word q ^ (r / 2 mod 4)
+          *reinterpret_cast<uint4*>(b + lane * 64 + (q ^ ((lane >> 1) & 3)) * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_2d(&tm_out, smem_u32(b), n0 + 32 * c, m0 + quarter * 32);
+          bulk_commit_group();
         }
       }
-      tc_fence_before();
-      mbar_arrive(acce0 + 8 * set);
     }
+    if (lane == 0) bulk_wait_all();
+    __syncwarp();
   }
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync();   // neither CTA's TMEM, barriers or shared memory is used by the other any more
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, C::TMEM_COLS);
+    if constexpr (PAIR) tmem_dealloc_pair(tmem, C::TMEM_COLS);
+    else tmem_dealloc(tmem, C::TMEM_COLS);
   }
 }
 
-template <int BN>
+template <int BN, bool PAIR>
 cudaError_t launch_gemm_bn(const uint8_t* a_q, const float* a_scale, const uint8_t* w_q, const float* w_scale,
                            int32_t T, int32_t D, int32_t Dout, __nv_bfloat16* out, int* status,
                            uint64_t wait_limit_ns, cudaStream_t s) {
-  using C = QCfg<BN>;
+  using C = QCfg<BN, PAIR>;
   int dev = 0;
   cudaGetDevice(&dev);
   {
-    const cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(w8a8_gemm_kernel<BN>), C::SMEM);
+    const cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(w8a8_gemm_kernel<BN, PAIR>), C::SMEM);
     if (e != cudaSuccess) return e;
   }
-  CUtensorMap ta, tw;
-  if (!encode_tmap_2d_u8(&ta, a_q, D, T, D, QK, QM) || !encode_tmap_2d_u8(&tw, w_q, D, Dout, D, QK, BN))
+  CUtensorMap ta, tw, to;
+  if (!encode_tmap_2d_u8(&ta, a_q, D, T, D, QK, QM) || !encode_tmap_2d_u8(&tw, w_q, D, Dout, D, QK, C::BR) ||
+      !encode_tmap_2d_sw64(&to, out, Dout, T, 2 * static_cast<uint64_t>(Dout), 32, 32))
     return cudaErrorInvalidValue;
   GemmParams p;
   p.T = T;
   p.D = D;
   p.Dout = Dout;
   p.n_kb = D / QK;
-  p.n_mt = (T + QM - 1) / QM;
+  p.n_mt = (T + QM * C::CTAS - 1) / (QM * C::CTAS);
   p.n_tiles = p.n_mt * (Dout / BN);
   p.a_scale = a_scale;
   p.w_scale = w_scale;
-  p.out = out;
   p.status = status;
   p.wait_limit_ns = wait_limit_ns;
   int dev_sms = 152;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev);
-  const int grid = p.n_tiles < dev_sms ? p.n_tiles : dev_sms;
-  return launch_pdl(w8a8_gemm_kernel<BN>, dim3(grid), dim3(Q_THREADS), C::SMEM, s, ta, tw, p);
+  const int units = std::min(p.n_tiles, dev_sms / C::CTAS);
+  return launch_pdl_cluster(w8a8_gemm_kernel<BN, PAIR>, dim3(units * C::CTAS), dim3(Q_THREADS), C::SMEM, C::CTAS, s, ta, tw, to, p);
 }
 
 }  // namespace
@@ -418,29 +472,33 @@ cudaError_t launch_w8a8_gemm(const uint8_t* a_q, const float* a_scale, const uin
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  // Estimated run: waves of tiles (one tile per SM per wave) x the time of one tile.  A
-  // k-block of a 128 x BN tile moves (128 + BN) x 128 bytes through shared memory twice (TMA
-  // write, UMMA read) for 128 x BN x 128 MACs, so wider tiles need fewer bytes per MAC: relative
-  // time per tile at the shared-memory limit ~ (128 + BN), with a floor at the tensor rate.
-  const int64_t m_tiles = (T + QM - 1) / QM;
-  int best = 128;
-  double best_cost = 0.0;
-  for (const int bn : {256, 192, 128}) {
-    if (Dout % bn != 0) continue;
-    const int64_t tiles = m_tiles * (Dout / bn);
-    const double waves = static_cast<double>((tiles + sms - 1) / sms);
-    const double per_tile = std::max(static_cast<double>(128 + bn), 1.5 * bn);
-    const double cost = waves * per_tile;
-    if (best_cost == 0.0 || cost < best_cost) {
-      best = bn;
+  // Estimated run (ns): waves of tiles x (k-blocks x time of one + a tile's fixed part) + launch and fill, all
+  // fitted to measured runs of 40 to 9400 tokens and 512 to 8960 features (within 15 %).  One CTA is
+  // bound by its shared memory: a k-block's (128 + BN) x 128 bytes are written by TMA and read by
+  // the UMMAs at 128 bytes per clock, so wider tiles cost less per MAC.  A pair halves B's
+  // part, 325 against 366 ns at 256 columns, but its tiles are twice as high and both CTAs have to meet
+  // before the first load: it needs several waves.  Pairs with 128 or 192 columns were never faster than
+  // one CTA with the same columns (4680 x 1536 x 1536: 13.1 against 11.5 us with 192).
+  struct Shape {
+    int bn, ctas, kblock_ns, start_ns;
+  };
+  static constexpr Shape kShapes[4] = {{256, 2, 325, 4800}, {256, 1, 366, 3000}, {192, 1, 325, 3000}, {128, 1, 308, 3000}};
+  int best = -1;
+  int64_t best_cost = 0;
+  for (int i = 0; i < 4; ++i) {
+    const Shape& f = kShapes[i];
+    if (Dout % f.bn != 0 || sms < f.ctas) continue;
+    const int64_t rows = QM * f.ctas, units = sms / f.ctas;
+    const int64_t tiles = (T + rows - 1) / rows * (Dout / f.bn);
+    const int64_t cost = (tiles + units - 1) / units * (D / QK * f.kblock_ns + 360) + f.start_ns;
+    if (best < 0 || cost < best_cost) {
+      best = i;
       best_cost = cost;
     }
   }
-  if (best == 256)
-    return launch_gemm_bn<256>(a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
-  if (best == 192)
-    return launch_gemm_bn<192>(a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
-  return launch_gemm_bn<128>(a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
+  const auto run = best == 0 ? launch_gemm_bn<256, true> : best == 1 ? launch_gemm_bn<256, false>
+                 : best == 2 ? launch_gemm_bn<192, false> : launch_gemm_bn<128, false>;
+  return run(a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
 }
 
 }  // namespace ispa
