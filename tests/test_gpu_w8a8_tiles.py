@@ -42,3 +42,17 @@ def test_rows_and_edges(T, D, Do):
     ref = qt.linear_w8a8(aq[rows], sa[rows], wq, sw)
     mag = (np.abs(qt.decode(aq[rows])) @ np.abs(qt.decode(wq)).T) * sa[rows][:, None].astype(np.float64) * sw.astype(np.float64)
     assert np.all(np.abs(y - ref) <= 2.0 ** -8 * np.abs(ref) + (D + 6) * 2.0 ** -24 * mag)
+
+
+@pytest.mark.parametrize("T,D", [(9, 16), (50, 1024), (33, 1040), (50, 1536), (21, 1552), (50, 2048), (17, 2064), (8, 3072),
+                                 (7, 3088), (3, 8960)])
+def test_quantised_rows_at_the_register_limits(T, D):
+    # rows that fill 4, 6, 8 and 12 words a lane exactly, or need a little more: codes and scales bit for bit
+    x = synth.bf16_round(np.random.default_rng(D).standard_normal((T, D), dtype=np.float32))
+    x[T // 2, D - 1] = 1e4
+    q = torch.empty(T, D, dtype=torch.uint8, device="cuda")
+    s = torch.empty(T, dtype=torch.float32, device="cuda")
+    abi.ispa_quantize_rows_e4m3(torch.from_numpy(x).to(torch.bfloat16).cuda(), T, D, q, s)
+    torch.cuda.synchronize()
+    rq, rs = qt.quantize_rows(synth.bf16_round(x))
+    assert np.array_equal(q.cpu().numpy(), rq) and np.array_equal(s.cpu().numpy(), rs)
