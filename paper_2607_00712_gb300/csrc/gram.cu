@@ -789,6 +789,22 @@ __global__ void __launch_bounds__(W_THREADS, 1)
   }
 }
 
+// CTAs of a call of `total` steps in tile passes of `len` steps (64 tokens) each.  The steps are cut evenly, so
+// with m CTAs for every pass each works on one tile; with one CTA per SM most CTAs get the end of one tile and
+// the beginning of another, a second read-back and flush worth `flush` steps.  Of the two the
+// one whose CTAs finish first, by a fit to measured runs (steps take 5 % longer on m CTAs a pass, whose flushes
+// come all at once).  Fewer CTAs than either never pay: a call of few tokens is bound by the read-backs and flushes that
+// a CTA does one after another, 5 us each for a 256 x 256 tile.  Before (16 steps or more for every CTA) and after, us:
+// D 1536 with 60 tokens 97 -> 13.0, 300 tokens 36 -> 15.8; D 512 with 1000 tokens 21.4 -> 14.9, 4680 tokens
+// 30.9 -> 21.9; D 2048 with 2000 tokens 42.6 -> 38.8; D 384 with 1000 tokens 15.2 -> 10.0.
+static int gram_grid(int64_t total, int64_t len, int sms, int flush) {
+  const int64_t passes = total / len;
+  if (passes > sms) return sms;
+  const int64_t m = sms / passes < len ? sms / passes : len;
+  const int64_t steps = (len + m - 1) / m;
+  return 21 * steps * sms < 20 * (total + flush * sms) ? static_cast<int>(passes * m) : sms;
+}
+
 static cudaError_t launch_gram_wide(int32_t D, int64_t T, int form, const void* op0, const void* op1,
                                     const void* op2, const float* unscale, float* gram, int* status,
                                     uint64_t wait_limit_ns, uint32_t* hb, cudaStream_t s) {
@@ -828,9 +844,7 @@ static cudaError_t launch_gram_wide(int32_t D, int64_t T, int form, const void* 
   int64_t total = 0;
   for (int k = 0; k < 3; ++k) total += static_cast<int64_t>(p.U[k]) * passes[k] * p.n_ktiles;
   if (total > INT32_MAX) return cudaErrorInvalidValue;
-  // one CTA per SM, each with at least 16 steps (a 1024-token run of one tile)
-  const int64_t want = (total + 15) / 16;
-  const int grid = static_cast<int>(want < sms ? (want > 0 ? want : 1) : sms);
+  const int grid = gram_grid(total, p.n_ktiles, sms, 9);
   p.tail_total = 0;
   for (int k = 0; k < 3; ++k) {
     p.waves[k] = p.U[k] / grid;
@@ -899,9 +913,7 @@ static cudaError_t launch_gram(int32_t D, int64_t T, int form, const void* op0, 
   p.status = status;
   p.wait_limit_ns = wait_limit_ns;
   p.heartbeat = hb;
-  // one CTA per SM, each with at least 16 steps (a 1024-token run of one tile)
-  const int64_t want = (total + 15) / 16;
-  const dim3 grid(static_cast<unsigned>(want < sms ? (want > 0 ? want : 1) : sms));
+  const dim3 grid(static_cast<unsigned>(gram_grid(total, p.n_ktiles, sms, 3)));
   return launch_pdl(gram_kernel<BN>, grid, dim3(G_THREADS), C::SMEM, s, tr[0], tr[1], tr[2], tc[0], tc[1], tc[2],
                     p);
 }
