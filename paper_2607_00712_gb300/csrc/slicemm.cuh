@@ -95,21 +95,29 @@ __device__ __forceinline__ int64_t sl_offset(int64_t chunk, int n_t, int r, int 
 }
 
 // The digits of eight fixed-point numbers as bf16, stored at dst + SL_BLOCK * slice (16 bytes each).
+// A number is rounded to 56 bits; with 128 added at every digit but the first its bytes are the digits plus 128
+// (the first keeps its sign and range [-128, 128]), so that a digit costs a byte permute and an addition: byte b under
+// the exponent of 2^23 is the fp32 number 2^23 + b.  Rounding and subtracting 64-bit digits one after another took five
+// times as many instructions: with fixed_to_double's funnel shifts a 1536 x 1536 solve 3.07 -> 2.93 ms, 5120 x 5120 28.4 -> 27.5.
 __device__ __forceinline__ void store_digits8(const int64_t* xi, uint8_t* dst) {
-  uint64_t r[8];
+  constexpr float kBias = 8388608.f + 128.f;
+  uint32_t lo[8], hi[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) r[i] = static_cast<uint64_t>(xi[i]);
+  for (int i = 0; i < 8; ++i) {
+    const uint64_t z = static_cast<uint64_t>(((xi[i] >> 7) + 1) >> 1) + 0x808080808080ull;   // no overflow at the top
+    lo[i] = static_cast<uint32_t>(z);
+    hi[i] = static_cast<uint32_t>(z >> 32);
+  }
 #pragma unroll
   for (int s = 0; s < SL; ++s) {
     uint32_t w[4];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int sh = 56 - 8 * s;
-      // round to nearest without overflow at the top: (r >> (sh - 1) + 1) >> 1
-      const int64_t d = ((static_cast<int64_t>(r[i]) >> (sh - 1)) + 1) >> 1;
-      r[i] -= static_cast<uint64_t>(d) << sh;
-      const uint32_t b = __float_as_uint(static_cast<float>(static_cast<int>(d))) >> 16;   // exact in bf16
-      w[i >> 1] = (i & 1) ? (w[i >> 1] | (b << 16)) : b;
+      uint32_t d;   // 2^23 + 128 + the digit
+      if (s == 0) d = 0x4B000080u + static_cast<uint32_t>(static_cast<int32_t>(hi[i]) >> 16);
+      else d = __byte_perm(s < 3 ? hi[i] : lo[i], 0x4B000000u, 0x7650u | static_cast<uint32_t>((6 - s) & 3));
+      const uint32_t b = __float_as_uint(__uint_as_float(d) - kBias);   // exact in bf16
+      w[i >> 1] = (i & 1) ? __byte_perm(w[i >> 1], b, 0x7632) : b;
     }
     *reinterpret_cast<uint4*>(dst + SL_BLOCK * s) = make_uint4(w[0], w[1], w[2], w[3]);
   }
@@ -304,27 +312,37 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 
-// (hi 2^32 + lo) 2^e rounded to nearest, without the fp64 pipe (2 operations per clock and SM); e is a row's and a column's exponent and a few tens: normal results only need the
-// integer path, the rest goes through ldexp.
+// (hi 2^32 + lo) 2^e rounded to nearest, without the fp64 pipe (2 operations per clock and SM); e is a row's and a
+// column's exponent and a few tens: normal results only need the integer path, in 32-bit words and funnel shifts, the rest goes
+// through ldexp.
 __device__ __forceinline__ double fixed_to_double(int64_t hi, uint32_t lo, int e) {
-  __int128 v = (static_cast<__int128>(hi) << 32) + lo;
-  const bool neg = v < 0;
-  unsigned __int128 a = neg ? -static_cast<unsigned __int128>(v) : static_cast<unsigned __int128>(v);
-  uint64_t top = static_cast<uint64_t>(a >> 64), low = static_cast<uint64_t>(a);
-  if ((top | low) == 0) return 0.0;
-  int shift = 64;                       // exponent of the word in `top`
-  if (top == 0) {
-    top = low;
-    low = 0;
-    shift = 0;
+  const uint32_t sign = static_cast<uint32_t>(static_cast<uint64_t>(hi) >> 32) & 0x80000000u;
+  const uint32_t neg = static_cast<uint32_t>(static_cast<int32_t>(sign) >> 31);   // all ones for a negative number
+  // magnitude: complement and add one
+  const uint32_t w0 = (lo ^ neg) - neg;
+  const uint64_t up = (static_cast<uint64_t>(hi) ^ (static_cast<uint64_t>(neg) << 32 | neg)) + (neg & (w0 == 0));
+  uint32_t x2 = static_cast<uint32_t>(up >> 32), x1 = static_cast<uint32_t>(up), x0 = w0;
+  int ex = 1023 + 95 + e;
+  if (x2 == 0) {   // the leading word first
+    x2 = x1;
+    x1 = x0;
+    x0 = 0;
+    ex -= 32;
+    if (x2 == 0) {
+      x2 = x1;
+      x1 = 0;
+      ex -= 32;
+      if (x2 == 0) return 0.0;
+    }
   }
-  const int lz = __clzll(static_cast<long long>(top));
-  uint64_t m = lz ? (top << lz) | (low >> (64 - lz)) : top;   // the leading 64 bits
-  const int ex = 1023 + 63 - lz + shift + e;
-  m = (m >> 11) + ((m >> 10) & 1);      // 53 bits; a carry out raises the exponent by itself
-  if (ex < 1 || ex > 2045) return ldexp(neg ? -static_cast<double>(m) : static_cast<double>(m), ex - 1023 - 52);
-  return __longlong_as_double(static_cast<long long>(((static_cast<uint64_t>(ex - 1) << 52) + m) |
-                                                     (neg ? 1ull << 63 : 0ull)));
+  const int lz = __clz(x2);
+  ex -= lz;
+  const uint32_t m1 = __funnelshift_l(x1, x2, lz), m0 = __funnelshift_l(x0, x1, lz);   // the leading 64 bits
+  // 53 bits; a carry out raises the exponent by itself
+  const uint64_t m = (static_cast<uint64_t>(m1 >> 11) << 32 | __funnelshift_r(m0, m1, 11)) + ((m0 >> 10) & 1);
+  if (ex < 1 || ex > 2045) return ldexp(sign ? -static_cast<double>(m) : static_cast<double>(m), ex - 1023 - 52);
+  return __hiloint2double(static_cast<int>((static_cast<uint32_t>(ex - 1) << 20) + static_cast<uint32_t>(m >> 32) + sign),
+                          static_cast<int>(static_cast<uint32_t>(m)));
 }
 
 __device__ __forceinline__ double pow2d(int e) {   // 2^e; 0 below the normal range, inf above it
@@ -351,6 +369,71 @@ __device__ __forceinline__ void sg_item(const SlGemm& p, bool tri, int t, int& r
   sg_tile(p, tri, tile, row, col);
   c0 = n_flush * piece / p.n_split * SG_FLUSH;
   c1 = min(n_flush * (piece + 1) / p.n_split * SG_FLUSH, p.n_chunks);
+}
+
+// The UMMAs of one chunk of 32 k (operands at da and db) into the eight sums, flush f: `first` and `last` chunk of it.
+__device__ __forceinline__ bool sg_umma_chunk(uint32_t tmem, uint64_t da, uint64_t db, bool first, bool last,
+                                              uint32_t gfull0, uint32_t gfree0, int f, const WaitCtx& wc) {
+#pragma unroll
+  for (int h = 0; h < 3; ++h) {
+    // the group's sums of the flush before have been read
+    if (first && !mbar_wait(gfree0 + 8 * h, (f & 1) ^ 1, wc, 43 + h, f)) return false;
+    tc_fence_after();
+#pragma unroll
+    for (int ks = 0; ks < SL_K / 16; ++ks)
+#pragma unroll
+      for (int i = 0; i < (h < 2 ? sg_s0(h + 1) : SL); ++i) {
+        // slice q of the rows with the columns' slices s0 .. s1 - 1 in one UMMA: sums q + s0 .. q + s1 - 1.
+        // The first one of a group starts all of its sums; in the last group that is q = 1 (q = 0 has none for s = 7)
+        const int q = h == 2 && i < 2 ? 1 - i : i;
+        const int s0 = sg_s0(h) > q ? sg_s0(h) - q : 0, s1 = sg_s0(h + 1) - q < SL ? sg_s0(h + 1) - q : SL;
+        umma_ss(tmem + 64 * (q + s0), da + (q * 2 * SL_BLOCK + ks * 256) / 16, db + (s0 * SL_BLOCK + ks * 256) / 16,
+                idesc_bf16(128, 64 * (s1 - s0), false, false), (!first || ks > 0 || i > 0) ? 1u : 0u);
+      }
+    if (last) tc_commit(gfull0 + 8 * h);
+  }
+  return true;
+}
+
+// Flush f's sums of this thread's row and SG_COLS columns (TMEM address tbase), added to hi 2^32 + lo in units of
+// 2^-70 of the rows' scales.  The whole warp calls it.
+__device__ __forceinline__ bool sg_read_sums(int64_t (&hi)[SG_COLS], uint32_t (&lo)[SG_COLS], uint32_t tbase, int lane,
+                                             uint32_t gfull0, uint32_t gfree0, int f, const WaitCtx& wc) {
+#pragma unroll
+  for (int h = 0; h < 3; ++h) {
+    if (!__all_sync(0xffffffffu, mbar_wait(gfull0 + 8 * h, f & 1, wc, 46 + h, f))) return false;
+    tc_fence_after();
+    const int ns = sg_s0(h + 1) - sg_s0(h);
+#pragma unroll
+    for (int c = 0; c < SG_COLS / 8; ++c) {
+      uint32_t v[3][8];
+#pragma unroll
+      for (int s = 0; s < ns; ++s) tmem_ld8(tbase + 64 * (sg_s0(h) + s) + 8 * c, v[s]);
+#pragma unroll
+      for (int s = 0; s < ns; ++s) tmem_wait_ld8(v[s]);
+      if (c == SG_COLS / 8 - 1) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(gfree0 + 8 * h);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int u0 = __float2int_rn(__uint_as_float(v[0][i])), u1 = __float2int_rn(__uint_as_float(v[1][i]));
+        const int u2 = ns > 2 ? __float2int_rn(__uint_as_float(v[2][i])) : 0;
+        if (h == 0) {
+          hi[8 * c + i] += static_cast<int64_t>(u0 * 256 + u1) * 65536 + static_cast<int64_t>(u2) * 256;   // |u0| <= 2^21
+        } else {
+          if (h == 1) hi[8 * c + i] += u0;
+          const int64_t l = h == 1 ? static_cast<int64_t>(u1) * (1 << 24)
+                                   : static_cast<int64_t>(u0) * 65536 + static_cast<int64_t>(u1) * 256 + u2;
+          const uint64_t sum = static_cast<uint64_t>(lo[8 * c + i]) + static_cast<uint32_t>(l);
+          lo[8 * c + i] = static_cast<uint32_t>(sum);
+          hi[8 * c + i] += (l >> 32) + static_cast<int64_t>(sum >> 32);
+        }
+      }
+    }
+  }
+  return true;
 }
 
 // 128 x 64 output tiles; TMEM holds the eight v_s of a tile (8 x 64 columns, s after s).  A stage is 32 k
@@ -439,28 +522,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(const SlGemm 
             }
             const uint64_t da = core_desc(sbase + st * SG_STAGE, 128, 512);
             const uint64_t db = core_desc(sbase + st * SG_STAGE + SG_A, 128, 512);
-#pragma unroll
-            for (int h = 0; h < 3; ++h) {
-              // the group's sums of the flush before have been read
-              if (c == c0 && !mbar_wait(gfree0 + 8 * h, (f & 1) ^ 1, wc, 43 + h, f)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-#pragma unroll
-              for (int ks = 0; ks < SL_K / 16; ++ks)
-#pragma unroll
-                for (int i = 0; i < (h < 2 ? sg_s0(h + 1) : SL); ++i) {
-                  // slice q of the rows with the columns' slices s0 .. s1 - 1 in one UMMA: sums q + s0 .. q + s1 - 1.
-                  // The first one of a group starts all of its sums; in the last group that is q = 1 (q = 0 has none for s = 7)
-                  const int q = h == 2 && i < 2 ? 1 - i : i;
-                  const int s0 = sg_s0(h) > q ? sg_s0(h) - q : 0, s1 = sg_s0(h + 1) - q < SL ? sg_s0(h + 1) - q : SL;
-                  umma_ss(tmem + 64 * (q + s0), da + (q * 2 * SL_BLOCK + ks * 256) / 16,
-                          db + (s0 * SL_BLOCK + ks * 256) / 16, idesc_bf16(128, 64 * (s1 - s0), false, false),
-                          (c > c0 || ks > 0 || i > 0) ? 1u : 0u);
-                }
-              if (c == c1 - 1) tc_commit(gfull0 + 8 * h);
-            }
+            ok = sg_umma_chunk(tmem, da, db, c == c0, c == c1 - 1, gfull0, gfree0, f, wc);
             if (ok) tc_commit(empty0 + 8 * st);
           }
         }
@@ -487,41 +549,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(const SlGemm 
       sg_item(p, TRI, t, row, col, k0, k1);
 #pragma unroll 1
       for (int c0 = k0; c0 < k1; c0 += SG_FLUSH, ++f) {
-#pragma unroll
-        for (int h = 0; h < 3; ++h) {
-          ok = ok && __all_sync(0xffffffffu, mbar_wait(gfull0 + 8 * h, f & 1, wc, 46 + h, f));
-          if (!ok) break;
-          tc_fence_after();
-          const int ns = sg_s0(h + 1) - sg_s0(h);
-#pragma unroll
-          for (int c = 0; c < SG_COLS / 8; ++c) {
-            uint32_t v[3][8];
-#pragma unroll
-            for (int s = 0; s < ns; ++s) tmem_ld8(tbase + 64 * (sg_s0(h) + s) + 8 * c, v[s]);
-#pragma unroll
-            for (int s = 0; s < ns; ++s) tmem_wait_ld8(v[s]);
-            if (c == SG_COLS / 8 - 1) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(gfree0 + 8 * h);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int u0 = __float2int_rn(__uint_as_float(v[0][i])), u1 = __float2int_rn(__uint_as_float(v[1][i]));
-              const int u2 = ns > 2 ? __float2int_rn(__uint_as_float(v[2][i])) : 0;
-              if (h == 0) {
-                hi[8 * c + i] += static_cast<int64_t>(u0 * 256 + u1) * 65536 + static_cast<int64_t>(u2) * 256;   // |u0| <= 2^21
-              } else {
-                if (h == 1) hi[8 * c + i] += u0;
-                const int64_t l = h == 1 ? static_cast<int64_t>(u1) * (1 << 24)
-                                         : static_cast<int64_t>(u0) * 65536 + static_cast<int64_t>(u1) * 256 + u2;
-                const uint64_t sum = static_cast<uint64_t>(lo[8 * c + i]) + static_cast<uint32_t>(l);
-                lo[8 * c + i] = static_cast<uint32_t>(sum);
-                hi[8 * c + i] += (l >> 32) + static_cast<int64_t>(sum >> 32);
-              }
-            }
-          }
-        }
+        ok = sg_read_sums(hi, lo, tbase, lane, gfull0, gfree0, f, wc);
         if (!ok) break;
       }
       if (!ok) break;
