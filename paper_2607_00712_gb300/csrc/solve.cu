@@ -344,7 +344,8 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
 // Inverse I of L's 128 x 128 diagonal blocks, fp64.  The factor is stored by columns and leaves the other half of
 // its array free: I_ij goes to [i][j], where column i has no L (the 64 x 64 blocks on the diagonal are
 // L's in `diag`).  One CTA per 8 columns of a block; thread (column, row group): right-looking substitution with its
-// rows in registers.
+// rows in registers.  The CTAs of all blocks' first columns, which have the longest chains, come first, and load only what they need: 117 -> 62 us at
+// 1536, 257 -> 151 at 5120.
 constexpr int IC = 8;
 constexpr int IG = 256 / IC;   // row groups
 constexpr int INV_SMEM = (TB * (TB + 1) + 2 * IC + TB) * 8;
@@ -356,11 +357,11 @@ __global__ void __launch_bounds__(256) inverse_kernel(const int64_t* fix, const 
   double* rd = xs + 2 * IC;                  // reciprocals of the diagonal
   pdl_wait();
   pdl_trigger();
-  const int b = blockIdx.y, c0 = blockIdx.x * IC, tid = threadIdx.x;
+  const int b = blockIdx.x, c0 = blockIdx.y * IC, tid = threadIdx.x;   // the first columns, most of the work, first
   constexpr double k63 = 1.0842021724855044e-19;   // 2^-63
   for (int e = tid; e < TB * TB; e += 256) {
     const int c = e >> 7, r = e & 127;
-    if (r < c) continue;
+    if (r < c || c < c0) continue;
     int64_t v;
     if ((c >> 6) == (r >> 6)) v = diag[(static_cast<int64_t>(2 * b + (c >> 6)) << 12) + ((c & 63) << 6) + (r & 63)];
     else v = fix[static_cast<int64_t>(b * TB + c) * Dp + b * TB + r];
@@ -619,7 +620,7 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     ISPA_CK(launch_slice_gemm<SL_CHOL>(p, sms, s));
   }
   double* inv = reinterpret_cast<double*>(w.fix);
-  ISPA_CK(launch_pdl(inverse_kernel, dim3(TB / IC, nb), dim3(256), INV_SMEM, s, static_cast<const int64_t*>(w.fix),
+  ISPA_CK(launch_pdl(inverse_kernel, dim3(nb, TB / IC), dim3(256), INV_SMEM, s, static_cast<const int64_t*>(w.fix),
                      static_cast<const int64_t*>(w.diag), Dp, inv));
   const int64_t ld = Dp;
   {
