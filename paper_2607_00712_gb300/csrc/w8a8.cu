@@ -197,13 +197,15 @@ struct QCfg {
 struct GemmParams {
   int32_t T, D, Dout, n_kb;
   int32_t n_mt, n_tiles;   // row tiles (of 256 rows for pairs); all tiles (tile t: rows (t % n_mt), columns (t / n_mt))
+  int32_t split;           // CTAs that share a tile's k-blocks (SPLIT)
   const float* a_scale;
   const float* w_scale;
+  __nv_bfloat16* out;
   int* status;
   uint64_t wait_limit_ns;
 };
 
-template <int BN, bool PAIR>
+template <int BN, bool PAIR, bool SPLIT>
 __global__ void __launch_bounds__(Q_THREADS, 1)
     w8a8_gemm_kernel(const __grid_constant__ CUtensorMap tm_a, const __grid_constant__ CUtensorMap tm_w,
                      const __grid_constant__ CUtensorMap tm_out, const GemmParams p) {
@@ -222,9 +224,12 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * QST, accf0 = empty0 + 8 * QST,
                  acce0 = accf0 + 16, drain_bar = acce0 + 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_kb = p.n_kb;
   const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
-  const int unit = blockIdx.x / C::CTAS, units = gridDim.x / C::CTAS;   // one CTA or pair per output tile
+  // one CTA, pair or (SPLIT) cluster per output tile
+  const int ctas = SPLIT ? p.split : C::CTAS, unit = blockIdx.x / ctas, units = gridDim.x / ctas;
+  // this CTA's k-blocks: of a split tile its share, else all
+  const int part = SPLIT ? static_cast<int>(cluster_ctarank()) : 0;
+  const int kb0 = SPLIT ? p.n_kb * part / p.split : 0, kb1 = SPLIT ? p.n_kb * (part + 1) / p.split : p.n_kb;
   // A pair's rank 0 issues the UMMAs: its full barriers count both CTAs' bytes, its set-empty barriers both
   // CTAs' epilogue warps.  The stage-empty, set-full and drain barriers are each CTA's own,
   // arrived at by commits that go to both.
@@ -272,7 +277,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
       bool ok = true;
       for (int t = unit; ok && t < p.n_tiles; t += units) {
         const int m0 = ((t % p.n_mt) * C::CTAS + rank) * QM, n0 = (t / p.n_mt) * BN;
-        for (int kb = 0; kb < n_kb; ++kb, ++g) {
+        for (int kb = kb0; kb < kb1; ++kb, ++g) {
           const int st = g % QST;
           if (!mbar_wait(empty0 + 8 * st, ((g / QST) & 1) ^ 1, wc, 31, g)) {
             ok = false;
@@ -311,7 +316,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
         if (!mbar_wait(acce0 + 8 * set, ((i >> 1) & 1) ^ 1, wc, 34, i)) break;
         tc_fence_after();
         const uint32_t acc = tmem + set * C::SET;
-        for (int kb = 0; kb < n_kb; ++kb, ++g) {
+        for (int kb = kb0; kb < kb1; ++kb, ++g) {
           const int st = g % QST;
           if (!mbar_wait(full0 + 8 * st, (g / QST) & 1, wc, 32, g)) {
             ok = false;
@@ -322,7 +327,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
           // four K=32 steps inside the 128-byte swizzle row (alternating chains for BN 128)
 #pragma unroll
           for (int k = 0; k < QK / 32; ++k) {
-            const uint32_t d = acc + (C::CHAINS == 2 ? (k & 1) * BN : 0), more = (kb > 0 || k >= C::CHAINS) ? 1u : 0u;
+            const uint32_t d = acc + (C::CHAINS == 2 ? (k & 1) * BN : 0), more = (kb > kb0 || k >= C::CHAINS) ? 1u : 0u;
             const uint64_t da = sw128_desc(sa + 32 * k, 16, 1024), db = sw128_desc(sb + 32 * k, 16, 1024);
             if constexpr (PAIR) umma_f8_pair(d, da, db, C::IDESC, more);
             else umma_f8(d, da, db, C::IDESC, more);
@@ -369,6 +374,23 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
         if constexpr (PAIR) mbar_arrive_cluster(cluster_map(acce0 + 8 * set, 0));
         else mbar_arrive(acce0 + 8 * set);
       }
+      if constexpr (SPLIT) {
+        // the partial sums into the stages, which have been read: 16-byte word q of row r at q ^ (r & 7)
+        float4* x = reinterpret_cast<float4*>(smem) + (quarter * 32 + lane) * (BN / 4);
+#pragma unroll
+        for (int c = 0; c < HC; ++c)
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            float s4[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              s4[e] = __uint_as_float(v[c][4 * q + e]);
+              if constexpr (C::CHAINS == 2) s4[e] += __uint_as_float(v[HC + c][4 * q + e]);
+            }
+            x[(half * (BN / 8) + 8 * c + q) ^ (lane & 7)] = make_float4(s4[0], s4[1], s4[2], s4[3]);
+          }
+        break;   // a split tile's CTA has no other
+      }
       if (m0 + quarter * 32 >= p.T) continue;   // uniform over the warp; rows past T inside the block are clipped
 #pragma unroll
       for (int c = 0; c < HC; ++c) {
@@ -405,6 +427,29 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
 
   tc_fence_before();
   __syncthreads();
+  if constexpr (SPLIT) {
+    cluster_sync();   // every CTA's partial sums are in its shared memory
+    static_assert(!SPLIT || BN == 128, "a row is four columns a lane");
+    const int m0 = unit % p.n_mt * QM, n0 = unit / p.n_mt * BN + 4 * lane;
+    const float4 sw = *reinterpret_cast<const float4*>(p.w_scale + n0);
+    // one warp per row of this CTA's share
+    for (int r = QM * part / p.split + warp; r < QM * (part + 1) / p.split && m0 + r < p.T; r += Q_THREADS / 32) {
+      const uint32_t x = sbase + (r * (BN / 4) + (lane ^ (r & 7))) * 16;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i = 0; i < p.split; ++i) {
+        const float4 v = cluster_ld4(cluster_map(x, i));
+        o.x += v.x;
+        o.y += v.y;
+        o.z += v.z;
+        o.w += v.w;
+      }
+      const float sa = p.a_scale[m0 + r];
+      *reinterpret_cast<uint2*>(p.out + static_cast<size_t>(m0 + r) * p.Dout + n0) =
+          make_uint2(pack_bf16x2(__fmul_rn(__fmul_rn(o.x, sa), sw.x), __fmul_rn(__fmul_rn(o.y, sa), sw.y)),
+                     pack_bf16x2(__fmul_rn(__fmul_rn(o.z, sa), sw.z), __fmul_rn(__fmul_rn(o.w, sa), sw.w)));
+    }
+    cluster_sync();   // no CTA leaves while another still reads its shared memory
+  }
   if constexpr (PAIR) cluster_sync();   // neither CTA's TMEM, barriers or shared memory is used by the other any more
   if (warp == 1) {
     tc_fence_after();
@@ -413,15 +458,15 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   }
 }
 
-template <int BN, bool PAIR>
-cudaError_t launch_gemm_bn(const uint8_t* a_q, const float* a_scale, const uint8_t* w_q, const float* w_scale,
+template <int BN, bool PAIR, bool SPLIT = false>
+cudaError_t launch_gemm_bn(int split, const uint8_t* a_q, const float* a_scale, const uint8_t* w_q, const float* w_scale,
                            int32_t T, int32_t D, int32_t Dout, __nv_bfloat16* out, int* status,
                            uint64_t wait_limit_ns, cudaStream_t s) {
   using C = QCfg<BN, PAIR>;
   int dev = 0;
   cudaGetDevice(&dev);
   {
-    const cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(w8a8_gemm_kernel<BN, PAIR>), C::SMEM);
+    const cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(w8a8_gemm_kernel<BN, PAIR, SPLIT>), C::SMEM);
     if (e != cudaSuccess) return e;
   }
   CUtensorMap ta, tw, to;
@@ -433,6 +478,8 @@ cudaError_t launch_gemm_bn(const uint8_t* a_q, const float* a_scale, const uint8
   p.D = D;
   p.Dout = Dout;
   p.n_kb = D / QK;
+  p.split = split;
+  p.out = out;
   p.n_mt = (T + QM * C::CTAS - 1) / (QM * C::CTAS);
   p.n_tiles = p.n_mt * (Dout / BN);
   p.a_scale = a_scale;
@@ -441,8 +488,8 @@ cudaError_t launch_gemm_bn(const uint8_t* a_q, const float* a_scale, const uint8
   p.wait_limit_ns = wait_limit_ns;
   int dev_sms = 152;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev);
-  const int units = std::min(p.n_tiles, dev_sms / C::CTAS);
-  return launch_pdl_cluster(w8a8_gemm_kernel<BN, PAIR>, dim3(units * C::CTAS), dim3(Q_THREADS), C::SMEM, C::CTAS, s, ta, tw, to, p);
+  const int ctas = SPLIT ? split : C::CTAS, units = SPLIT ? p.n_tiles : std::min(p.n_tiles, dev_sms / ctas);
+  return launch_pdl_cluster(w8a8_gemm_kernel<BN, PAIR, SPLIT>, dim3(units * ctas), dim3(Q_THREADS), C::SMEM, ctas, s, ta, tw, to, p);
 }
 
 }  // namespace
@@ -489,6 +536,7 @@ cudaError_t launch_w8a8_gemm(const uint8_t* a_q, const float* a_scale, const uin
     int bn, ctas, kblock_ns, start_ns;
   };
   static constexpr Shape kShapes[4] = {{256, 2, 325, 4800}, {256, 1, 366, 3000}, {192, 1, 325, 3000}, {128, 1, 308, 3000}};
+  const int64_t m_tiles = (static_cast<int64_t>(T) + QM - 1) / QM;
   int best = -1;
   int64_t best_cost = 0;
   for (int i = 0; i < 4; ++i) {
@@ -502,9 +550,25 @@ cudaError_t launch_w8a8_gemm(const uint8_t* a_q, const float* a_scale, const uin
       best_cost = cost;
     }
   }
+  // Few tiles and many k-blocks: clusters of `split` CTAs share a tile's k-blocks and merge their sums through distributed
+  // shared memory, 2.6 to 2.9 us more for two cluster barriers and the merge.  64 x 5120 -> 640: 14.3 -> 6.3 us, 256 x 5120
+  // -> 1536: 14.7 -> 8.6, 40 x 1536 -> 1536: 6.4 -> 6.0; 512 x 2048 -> 2048 stays whole (7.97 against 8.54).  As
+  // many clusters as run at once: of four or eight CTAs that is about four fifths of the chip.
+  int split = 1;
+  for (const int c : {2, 4, 8}) {
+    const int64_t tiles = m_tiles * (Dout / 128);
+    if (D / QK < c || tiles * c * (c > 2 ? 5 : 4) > 4 * static_cast<int64_t>(sms)) break;
+    const int64_t cost = (D / QK + c - 1) / c * 308 + 360 + 3000 + 2500 + 50 * c;
+    if (cost < best_cost) {
+      split = c;
+      best_cost = cost;
+    }
+  }
+  if (split > 1)
+    return launch_gemm_bn<128, false, true>(split, a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
   const auto run = best == 0 ? launch_gemm_bn<256, true> : best == 1 ? launch_gemm_bn<256, false>
                  : best == 2 ? launch_gemm_bn<192, false> : launch_gemm_bn<128, false>;
-  return run(a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
+  return run(1, a_q, a_scale, w_q, w_scale, T, D, Dout, o, status, wait_limit_ns, s);
 }
 
 }  // namespace ispa

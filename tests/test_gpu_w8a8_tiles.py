@@ -56,3 +56,10 @@ def test_quantised_rows_at_the_register_limits(T, D):
     torch.cuda.synchronize()
     rq, rs = qt.quantize_rows(synth.bf16_round(x))
     assert np.array_equal(q.cpu().numpy(), rq) and np.array_equal(s.cpu().numpy(), rs)
+
+
+# few tiles: 8, 4 and 2 CTAs share a tile's k-blocks, evenly or not; the last row tile is ragged
+@pytest.mark.parametrize("T,D,Do", [(40, 1536, 1536), (1, 5120, 128), (129, 4736, 256), (52, 4224, 2048), (300, 2688, 768),
+                                    (128, 5120, 5120), (200, 3200, 4096)])
+def test_split_contractions(T, D, Do):
+    test_rows_and_edges(T, D, Do)
