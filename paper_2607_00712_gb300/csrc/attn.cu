@@ -51,9 +51,7 @@
 #include <stdint.h>
 
 #include <algorithm>
-#include <map>
-#include <mutex>
-#include <tuple>
+#include <atomic>
 
 #include "internal.h"
 #include "pdl.cuh"
@@ -995,16 +993,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
 }
 
-// Clusters of c CTAs of this kernel that the device holds at once (asked once per device and kernel).
+// Clusters of c CTAs of this kernel that the device holds at once.
 static int max_clusters(const void* func, int c, int smem) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, const void*, int>, int> known;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  std::lock_guard<std::mutex> lock(mu);
-  const auto key = std::make_tuple(dev, func, c);
-  const auto it = known.find(key);
-  if (it != known.end()) return it->second;
+  if (set_smem_limit_once(func, smem) != cudaSuccess) return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(c));
   cfg.blockDim = dim3(NTHREADS);
@@ -1020,7 +1011,6 @@ static int max_clusters(const void* func, int c, int smem) {
     cudaGetLastError();
     n = 0;
   }
-  known[key] = n;
   return n;
 }
 
@@ -1042,6 +1032,7 @@ static SplitPlan split_plan(int items, int n_tiles, int sms, F&& clusters) {
   SplitPlan best{0, 1};
   int cost = n_tiles - n_tiles / 10;
   for (int c = 2; r > 0 && c <= 8 && 2 * c <= n_tiles; ++c) {
+    if ((n_tiles + c - 1) / c + 5 >= cost) continue;   // not even in one round
     const int n = clusters(c);
     if (n <= 0) continue;
     const int rounds = (r + n - 1) / n;
@@ -1069,16 +1060,21 @@ static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, cons
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(whole), C::SMEM);
   if (e != cudaSuccess) return e;
-  e = set_smem_limit_once(reinterpret_cast<const void*>(split), Cfg<HD, QK8, false>::SMEM);
-  if (e != cudaSuccess) return e;
   p.n_qt = (p.n_q + BM - 1) / BM;
   const int64_t all = static_cast<int64_t>(p.n_qt) * p.num_heads;
   if (all > INT32_MAX) return cudaErrorInvalidValue;
   const int items = static_cast<int>(all);
   SplitPlan plan{0, 1};
-  if (!PV8 && !p.dual)
-    plan = split_plan(items, p.n_tiles, sms,
-                      [&](int c) { return max_clusters(reinterpret_cast<const void*>(split), c, C::SMEM); });
+  if (!PV8 && !p.dual) {
+    static std::atomic<int> known[8][9];   // per device and cluster size, plus one: asked once
+    plan = split_plan(items, p.n_tiles, sms, [&](int c) {
+      const int k = dev < 8 ? known[dev][c].load(std::memory_order_relaxed) : 0;
+      if (k > 0) return k - 1;
+      const int n = max_clusters(reinterpret_cast<const void*>(split), c, Cfg<HD, QK8, false>::SMEM);
+      if (dev < 8) known[dev][c].store(n + 1, std::memory_order_relaxed);
+      return n;
+    });
+  }
   const int first = items - plan.items;
   p.item0 = 0;
   p.wait_first = 1;
@@ -1087,6 +1083,8 @@ static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, cons
     if (e != cudaSuccess) return e;
   }
   if (plan.items > 0) {
+    e = set_smem_limit_once(reinterpret_cast<const void*>(split), Cfg<HD, QK8, false>::SMEM);
+    if (e != cudaSuccess) return e;
     p.item0 = first;
     p.wait_first = first == 0;
     cudaLaunchConfig_t cfg = {};
