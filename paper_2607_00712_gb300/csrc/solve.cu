@@ -14,8 +14,8 @@
 // products with the inverses of L's 128 x 128 diagonal blocks, and tr(W^T S W) = sum_ij S_ij (W W^T)_ij, half
 // the work of S W and nothing to store.  Plain fp64 code ran all of it at 1.09 TFLOP/s, the chip's
 // fp64 rate: 782 ms at hidden 5120 and 33 ms at 1536 (where the panels' launches and latency counted
-// too), against 27.5 and 2.93 ms.  What bounds it now: at 5120 the products' tensor time and read-back (22
-// of 28 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
+// too), against 27.5 and 2.90 ms.  What bounds it now: at 5120 the products' tensor time and read-back (21
+// of 27 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
 // dW's error against 64-bit arithmetic (before its rounding to fp32) is 0.4 to 0.8 times the plain code's.
 //
 // The factorisation runs in fixed point.  Row and column i are scaled by a power of two (exactly)
