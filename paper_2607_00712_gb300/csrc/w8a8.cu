@@ -346,6 +346,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     constexpr int HC = BN / 64;   // 32-column chunks of this warp's half
     const int quarter = warp & 3, half = (warp - 2) >> 2;
     uint8_t* block = smem + C::OFF_OUT + (warp - 2) * 2 * Q_BLOCK;
+    int first = 0;   // block of the tile's first store: they alternate on across tiles, also when a tile has three
     int i = 0;
     for (int t = unit; t < p.n_tiles; t += units, ++i) {
       const int set = i & 1;
@@ -394,8 +395,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
       if (m0 + quarter * 32 >= p.T) continue;   // uniform over the warp; rows past T inside the block are clipped
 #pragma unroll
       for (int c = 0; c < HC; ++c) {
-        uint8_t* b = block + (c & 1) * Q_BLOCK;
-        if (lane == 0) bulk_wait_read<1>();   // the store before last has read this block
+        uint8_t* b = block + ((first + c) & 1) * Q_BLOCK;
+        if (lane == 0) bulk_wait_read<1>();   // the store before last, this block's last, has read it
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -420,6 +421,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
           bulk_commit_group();
         }
       }
+      first ^= HC & 1;
     }
     if (lane == 0) bulk_wait_all();
     __syncwarp();
