@@ -492,8 +492,8 @@ ISPA_API ispa_status ispa_ls_accumulate_ex(ispa_ls_state* state, const void* a_l
 ISPA_API size_t ispa_ls_solve_workspace_size(int32_t dim, int32_t d_out);
 
 /*
- * Closed-form absorption (Eq. 5) and feasibility score (Eq. 6), with the accuracy of fp64
- * arithmetic (products of fp64-grade operands by exact slices on the tensor cores):
+ * Closed-form absorption (Eq. 5) and feasibility score (Eq. 6), fp64-grade (products on the
+ * tensor cores by exact slices; see Accuracy below):
  *   dW  = (G + lambda I)^{-1} X W          (Cholesky solve, Eq. 5 with R = Delta W)
  *   eps = || A_loc (W + dW) - A_full W ||_F^2
  *       = tr(W^T S W) - ||L^{-1} X W||_F^2 - lambda ||dW||_F^2,  L L^T = G + lambda I.
@@ -502,6 +502,12 @@ ISPA_API size_t ispa_ls_solve_workspace_size(int32_t dim, int32_t d_out);
  *   dW      : fp32 [dim][d_out] output
  *   eps_out : HOST double (nullable)
  *   lambda  : ridge weight on the unnormalised sums (paper default 1e-3)
+ * Accuracy, before dW's rounding to fp32: operands keep 56 bits below the largest value of their
+ * row or column, after exact scalings by powers of two that give
+ * M = G + lambda I a diagonal near 1 and X's columns one size.  So row i of X W is off by at most
+ * dim 2^-54 sqrt(M_ii) max_j (sqrt(S_jj) |W_jk|), where fp64 arithmetic has
+ * dim 2^-53 sum_j |X_ij W_jk|, and what the factorisation and the solves lose is a perturbation of
+ * M_ij small against sqrt(M_ii M_jj), as in an fp64 Cholesky solve.
  * Synchronises `stream`.  Errors: ISPA_ERR_NOT_SPD if a Cholesky pivot is not
  * positive (dW and eps are then meaningless); ISPA_ERR_TIMEOUT if a device wait ran out.
  */

@@ -44,7 +44,7 @@ constexpr int SL_NAN = 1 << 28;             // exponent of a row that holds a Na
 // only (the fp64 pipe converts 2 numbers per clock and SM).
 __device__ __forceinline__ int64_t fix63(uint64_t mant, int shift, bool neg) {   // mant * 2^shift
   uint64_t v;
-  if (shift >= 0) v = mant << shift;
+  if (shift >= 0) v = mant << (shift & 63);   // below 64 for all but zero
   else v = shift > -63 ? (mant + (1ull << (-shift - 1))) >> -shift : 0ull;
   return neg ? -static_cast<int64_t>(v) : static_cast<int64_t>(v);
 }
@@ -141,6 +141,9 @@ struct SliceParams {
                        // a window's segments start again at the op's first chunk
   int32_t lower;       // z_k segments: 1: only the rows past the segment's k, -1: only those before them
   int32_t n_t;         // tiles of 64 rows of the op
+  const int32_t* k_exp;   // SCALED: value k of a row is taken times 2^(k_sign k_exp[k]); k_sign is 1 or -1
+  int32_t k_sign;
+  const int32_t* r_max;   // SCALED, row-contiguous source: the rows' exponents (SL_NONE, SL_NAN as SliceMax takes them)
   uint8_t* op;
   int32_t* exps;
 };
@@ -155,6 +158,38 @@ __device__ __forceinline__ int sl_row0(const SliceParams& p, int z) { return p.w
 __device__ __forceinline__ int sl_pad(const SliceParams& p, int ks) {
   return p.z_k ? (ks + SL_K - 1) / SL_K * SL_K : p.k_pad;
 }
+// The largest magnitude of a row, and its exponent.  SCALED compares exponents instead: a power of two for each value
+// makes the magnitudes leave their type, and the row's exponent is all that is taken from them.
+constexpr int SL_NONE = -(1 << 30);   // no value yet, or all zero
+template <typename T, bool SCALED>
+struct SliceMax {
+  using V = typename SliceSrc<T>::Mag;
+  static constexpr V none = 0;
+  static __device__ V of(T x, int) { return SliceSrc<T>::mag(x); }
+  static __device__ int exp_of(V v) { return SliceSrc<T>::exp_of(v); }
+};
+template <typename T>
+struct SliceMax<T, true> {
+  using V = int;
+  static constexpr V none = SL_NONE;
+  static __device__ V of(T x, int scale) {
+    const typename SliceSrc<T>::Mag m = SliceSrc<T>::mag(x);
+    return m == 0 ? SL_NONE : SliceSrc<T>::exp_of(m) + scale;
+  }
+  static __device__ int exp_of(V v) { return v == SL_NONE ? 0 : (v > SL_NAN / 2 ? SL_NAN : v); }
+};
+// The scales of values k .. k + 7 (k % 8 == 0; k_exp is 16-byte aligned and goes up to k_pad).
+template <bool SCALED>
+__device__ __forceinline__ void sl_scales8(const SliceParams& p, int k, int (&s)[8]) {
+  int4 a = make_int4(0, 0, 0, 0), b = a;
+  if constexpr (SCALED) {
+    a = reinterpret_cast<const int4*>(p.k_exp + k)[0];
+    b = reinterpret_cast<const int4*>(p.k_exp + k)[1];
+  }
+  s[0] = p.k_sign * a.x, s[1] = p.k_sign * a.y, s[2] = p.k_sign * a.z, s[3] = p.k_sign * a.w;
+  s[4] = p.k_sign * b.x, s[5] = p.k_sign * b.y, s[6] = p.k_sign * b.z, s[7] = p.k_sign * b.w;
+}
+
 // Which of a segment's values are there (the others are taken as zero): all, k <= row, or k >= row.
 enum SlTri : int { SL_FULL, SL_LOWER, SL_UPPER };
 template <int TRI>
@@ -167,12 +202,13 @@ __device__ __forceinline__ bool sl_there(int row, int k) {
 // thread 8 k of one row, a warp 8 rows x 32 k, so that each slice of it is one contiguous 512-byte
 // store.  (Loading once, in the second pass's order, and reducing over the CTA is slower, 10.1 us
 // against 9.1 on average in a 5120 x 5120 solve: each of those loads touches 32 sectors.)
-template <typename T, int TRI>
+template <typename T, int TRI, bool SCALED>
 __global__ void __launch_bounds__(512) slice_rows_kernel(const SliceParams p) {
   using S = SliceSrc<T>;
+  using M = SliceMax<T, SCALED>;
   pdl_wait();
   pdl_trigger();
-  __shared__ typename S::Mag red[2][8];
+  __shared__ typename M::V red[2][8];
   const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
   const int zc = sl_z(p, z), r0 = sl_row0(p, z) + blockIdx.x * 8;
   if (p.lower > 0 && r0 < (z + 1) * p.k_pad) return;
@@ -180,13 +216,13 @@ __global__ void __launch_bounds__(512) slice_rows_kernel(const SliceParams p) {
   const int rows = sl_rows(p, z), ks = sl_ks(p, z), k_pad = sl_pad(p, ks);
   if (p.rows_total && r0 >= rows) return;
   const T* src = static_cast<const T*>(p.src) + z * p.z_src + r0 * p.ld;
-  typename S::Mag m = 0;
+  typename M::V m = M::none;
   {
     const int r = warp & 7;
     const T* row = src + r * p.ld;
     if (r0 + r < rows) {
       for (int k = lane + 32 * (warp >> 3); k < ks; k += 4 * n_warp)
-        if (sl_there<TRI>(r0 + r, k)) m = max(m, S::mag(row[k]));
+        if (sl_there<TRI>(r0 + r, k)) m = max(m, M::of(row[k], SCALED ? p.k_sign * p.k_exp[k] : 0));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -195,16 +231,18 @@ __global__ void __launch_bounds__(512) slice_rows_kernel(const SliceParams p) {
   __syncthreads();
   const int r = lane & 7, kc = lane >> 3;
   m = n_warp > 8 ? max(red[0][r], red[1][r]) : red[0][r];
-  const int E = S::exp_of(m);
+  const int E = M::exp_of(m);
   if (threadIdx.x < 8) p.exps[zc * p.z_exp + z * p.z_rows + r0 + r] = E;
   const bool live = r0 + r < rows && E != SL_NAN;
   const T* row = src + r * p.ld;
   for (int c = warp; c < k_pad / SL_K; c += n_warp) {
     int64_t xi[8];
+    int scale[8];
+    sl_scales8<SCALED>(p, c * SL_K + kc * 8, scale);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = c * SL_K + kc * 8 + i;
-      xi[i] = live && k < ks && sl_there<TRI>(r0 + r, k) ? S::fixed(row[k], E) : 0;
+      xi[i] = live && k < ks && sl_there<TRI>(r0 + r, k) ? S::fixed(row[k], E - scale[i]) : 0;
     }
     store_digits8(xi, p.op + sl_offset(zc * (p.z_k / SL_K) + c, p.n_t, z * p.z_rows + r0 + r, kc));
   }
@@ -213,13 +251,14 @@ __global__ void __launch_bounds__(512) slice_rows_kernel(const SliceParams p) {
 // Source with rows contiguous (k strided).  One CTA (8 warps, 32 for long segments) per 32 rows and
 // segment; lane = row, so every load is a contiguous run of the source and every slice store four
 // 128-byte runs.  Where that leaves SMs idle the stores are split over blockIdx.z, each CTA finding the exponents
-// for itself: 57 -> 21 us for a 1536 x 1536 W.
-template <typename T, int TRI>
+// for itself (SCALED: they are given, six times over the search took as long as the stores).
+template <typename T, int TRI, bool SCALED>
 __global__ void __launch_bounds__(1024) slice_cols_kernel(const SliceParams p) {
   using S = SliceSrc<T>;
+  using M = SliceMax<T, SCALED>;
   pdl_wait();
   pdl_trigger();
-  __shared__ typename S::Mag red[32][32];
+  __shared__ typename M::V red[32][32];
   const int z = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
   const int zc = sl_z(p, z), r0 = sl_row0(p, z) + blockIdx.x * 32, r = r0 + lane;
   if (p.lower > 0 && r0 < (z + 1) * p.k_pad) return;
@@ -228,25 +267,35 @@ __global__ void __launch_bounds__(1024) slice_cols_kernel(const SliceParams p) {
   if (p.rows_total && r0 >= rows) return;
   const T* src = static_cast<const T*>(p.src) + z * p.z_src + r;
   const bool in = r < rows;
-  typename S::Mag m = 0;
-  if (in) {
-#pragma unroll 8
-    for (int k = warp; k < ks; k += n_warp)
-      if (sl_there<TRI>(r, k)) m = max(m, S::mag(src[k * p.ld]));
+  typename M::V m = M::none;
+  if constexpr (SCALED) {
+    if (in) m = p.r_max[r];
+  } else {
+    if (in) {
+      for (int q = warp; 8 * q < ks; q += n_warp) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int k = 8 * q + i;
+          if (k < ks && sl_there<TRI>(r, k)) m = max(m, M::of(src[k * p.ld], 0));
+        }
+      }
+    }
+    red[warp][lane] = m;
+    __syncthreads();
+    for (int w = 0; w < n_warp; ++w) m = max(m, red[w][lane]);
   }
-  red[warp][lane] = m;
-  __syncthreads();
-  for (int w = 0; w < n_warp; ++w) m = max(m, red[w][lane]);
-  const int E = S::exp_of(m);
+  const int E = M::exp_of(m);
   if (z * p.z_rows + r >= p.n_t * 64) return;
   if (warp == 0 && blockIdx.z == 0) p.exps[zc * p.z_exp + z * p.z_rows + r] = E;
   const bool live = in && E != SL_NAN;
   for (int q = warp + n_warp * blockIdx.z; q < k_pad / 8; q += n_warp * gridDim.z) {
     int64_t xi[8];
+    int scale[8];
+    sl_scales8<SCALED>(p, 8 * q, scale);
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int k = 8 * q + i;
-      xi[i] = live && k < ks && sl_there<TRI>(r, k) ? S::fixed(src[k * p.ld], E) : 0;
+      xi[i] = live && k < ks && sl_there<TRI>(r, k) ? S::fixed(src[k * p.ld], E - scale[i]) : 0;
     }
     store_digits8(xi, p.op + sl_offset(zc * (p.z_k / SL_K) + (q >> 2), p.n_t, z * p.z_rows + r, q & 3));
   }

@@ -16,7 +16,9 @@
 // fp64 rate: 782 ms at hidden 5120 and 33 ms at 1536 (where the panels' launches and latency counted
 // too), against 27.5 and 2.90 ms.  What bounds it now: at 5120 the products' tensor time and read-back (21
 // of 27 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
-// dW's error against 64-bit arithmetic (before its rounding to fp32) is 0.4 to 0.8 times the plain code's.
+// dW's error against 80-bit arithmetic, before its rounding to fp32, was 0.03 to 0.9 times the plain code's (dim 384,
+// five draws each): features of one size or spread by exp(2 N(0, 1)) 0.3 to 0.4, rank-deficient sums 0.6, rank 20 plus
+// noise 0.14, near-duplicate pairs 0.26, singular values falling to 1e-4 0.9; scaled condition numbers 13 to 3e7.
 //
 // The factorisation runs in fixed point.  Row and column i are scaled by a power of two (exactly)
 // so that M_ii lies in [1/4, 1); then every |M_ij|, every element of every Schur complement and
@@ -51,11 +53,15 @@ constexpr int PR = 32;     // panel rows per CTA
 constexpr int FLAG_NOT_SPD = 1;
 
 // t_i: the power of two with M_ii 2^(-2 t_i) in [1/4, 1).  Rows past D (padding) get 0.
+// u, ew: where col_exp_kernel's maxima start.
+constexpr int U_NONE = -(1 << 20);   // a column of zeros: its weights count for nothing
 __global__ void __launch_bounds__(256) equil_kernel(const float* __restrict__ gram, int D, int Dp, double lambda,
-                                                    int32_t* __restrict__ t, int* flag) {
+                                                    int32_t* __restrict__ t, int32_t* __restrict__ u, int n,
+                                                    int32_t* __restrict__ ew, int* flag) {
   pdl_wait();
   pdl_trigger();
   const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i < n) ew[i] = SL_NONE;
   if (i >= Dp) return;
   int e = 0;
   if (i < D) {
@@ -67,6 +73,43 @@ __global__ void __launch_bounds__(256) equil_kernel(const float* __restrict__ gr
     }
   }
   t[i] = e;
+  u[i] = U_NONE;
+}
+
+// out[j] = max(out[j], exponent of max_i |m[i][j]| 2^(sign add[i])) for the columns of an fp32 matrix.  NANS: SL_NAN
+// for a column that isn't finite (else such values are passed over).  A CTA takes 64 columns x 64 rows.
+//
+// It gives u_j, the power of two with max_i |X_ij| 2^(-t_i - u_j) in [1/2, 1), and the columns' exponents of
+// 2^(u_j) W_jk.  X W is formed from X_ij 2^(-u_j) and W_jk 2^(u_j): both operands keep 56 bits below the largest value
+// of a row or a column, so what counts is that the features j meet there at one size.  Without it a W that undoes
+// large differences between features (W_j ~ 1 / f_j) lost as many bits as they differ by: dW's error at dim 384 was
+// 7e-11 with f = exp(3 N(0, 1)) and 1e-7 with exp(4 N(0, 1)), where it is 4e-16 now and fp64 code has 1e-15.  The two
+// launches and the scales cost 11 us of 2.91 ms at 1536 x 1536, 85 us of 27.5 ms at 5120 x 5120.
+constexpr int U_COLS = 64, U_ROWS = 64, U_PART = U_ROWS / (256 / U_COLS);
+template <bool NANS>
+__global__ void __launch_bounds__(256) col_exp_kernel(const float* __restrict__ m, int64_t ld, int rows, int cols,
+                                                      const int32_t* __restrict__ add, int sign,
+                                                      int32_t* __restrict__ out) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ int red[256];
+  const int j = blockIdx.x * U_COLS + threadIdx.x % U_COLS;
+  const int i0 = blockIdx.y * U_ROWS + threadIdx.x / U_COLS * U_PART;
+  int e = SL_NONE;
+#pragma unroll
+  for (int n = 0; n < U_PART; ++n) {
+    const int i = i0 + n;
+    if (i >= rows || j >= cols) continue;
+    const uint32_t mag = SliceSrc<float>::mag(m[i * ld + j]);
+    const int xe = SliceSrc<float>::exp_of(mag);
+    if (mag != 0 && (NANS || xe != SL_NAN)) e = max(e, xe == SL_NAN ? SL_NAN : xe + sign * add[i]);
+  }
+  red[threadIdx.x] = e;
+  __syncthreads();
+  if (threadIdx.x >= U_COLS || j >= cols) return;
+#pragma unroll
+  for (int n = 1; n < 256 / U_COLS; ++n) e = max(e, red[threadIdx.x + n * U_COLS]);
+  if (e != SL_NONE) atomicMax(out + j, e);
 }
 
 // fix[j][i] (i >= j) = M_ij 2^(-t_i - t_j) with 62 fraction bits, from G's upper triangle (row j of G is column
@@ -451,7 +494,7 @@ struct SolveWs {
   double* B;               // by columns [d_out][Dp]: X W, then Y, then Z
   uint8_t *op_panel, *op_s, *op_n, *op_i, *op_it;
   int64_t* diag;
-  int32_t *t, *ea, *en, *eb, *es, *ei, *eit;
+  int32_t *t, *u, *ew, *ea, *en, *eb, *es, *ei, *eit;
   double* scal;            // [0] ||Y||^2, [1] ||dW||^2, [2] tr(W^T S W)
   int* flag;
   size_t bytes;
@@ -486,6 +529,8 @@ SolveWs carve(void* ws, int D, int d_out) {
   w.op_it = take(TB / SL_K * chunk_d);
   w.diag = reinterpret_cast<int64_t*>(take(Dp * NB * 8));
   w.t = reinterpret_cast<int32_t*>(take(Dp * 4));
+  w.u = reinterpret_cast<int32_t*>(take(Dp * 4));
+  w.ew = reinterpret_cast<int32_t*>(take(static_cast<size_t>(d_out) * 4));
   w.ea = reinterpret_cast<int32_t*>(take((Dp + w.win - 1) / w.win * Dp * 4));
   w.en = reinterpret_cast<int32_t*>(take(w.win / TB * Dp * 4));
   w.eb = reinterpret_cast<int32_t*>(take(static_cast<size_t>(w.np) * 4));
@@ -513,19 +558,19 @@ SliceParams slice(const void* src, int64_t ld, int rows, int ks, int k_pad, int 
 }
 
 // grid_rows: rows of a segment in the op (multiples of 8, those past the valid ones are zeroed).
-template <typename T, int TRI = SL_FULL>
+template <typename T, int TRI = SL_FULL, bool SCALED = false>
 cudaError_t slice_rows(const SliceParams& p, int grid_rows, int n_seg, cudaStream_t s) {
   const dim3 grid(grid_rows / 8, n_seg);
-  return launch_pdl(slice_rows_kernel<T, TRI>, grid, dim3(p.k_pad > 512 ? 512 : 256), 0, s, p);
+  return launch_pdl(slice_rows_kernel<T, TRI, SCALED>, grid, dim3(p.k_pad > 512 ? 512 : 256), 0, s, p);
 }
 
-template <typename T, int TRI = SL_FULL>
+template <typename T, int TRI = SL_FULL, bool SCALED = false>
 cudaError_t slice_cols(const SliceParams& p, int grid_rows, int n_seg, cudaStream_t s) {
   dim3 grid((grid_rows + 31) / 32, n_seg);
   const int warps = p.k_pad > 128 ? 32 : 8, most = p.k_pad / 8 / warps;   // parts with work for every warp
   const int fill = 304 / static_cast<int>(grid.x * grid.y);
   grid.z = fill < 1 || most < 1 ? 1 : (fill < most ? fill : most);
-  return launch_pdl(slice_cols_kernel<T, TRI>, grid, dim3(32 * warps), 0, s, p);
+  return launch_pdl(slice_cols_kernel<T, TRI, SCALED>, grid, dim3(32 * warps), 0, s, p);
 }
 
 }  // namespace
@@ -554,7 +599,13 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
   ISPA_CK(set_smem_limit_once(reinterpret_cast<const void*>(inverse_kernel), INV_SMEM));
   ISPA_CK(set_smem_limit_once(reinterpret_cast<const void*>(panel_kernel), PANEL_SMEM));
   ISPA_CK(cudaMemsetAsync(w.scal, 0, 256, s));
-  ISPA_CK(launch_pdl(equil_kernel, dim3((Dp + 255) / 256), dim3(256), 0, s, gram, D, Dp, lambda, w.t, w.flag));
+  ISPA_CK(launch_pdl(equil_kernel, dim3(((Dp > d_out ? Dp : d_out) + 255) / 256), dim3(256), 0, s, gram, D, Dp, lambda,
+                     w.t, w.u, d_out, w.ew, w.flag));
+  auto col_grid = [&](int cols) { return dim3((cols + U_COLS - 1) / U_COLS, (D + U_ROWS - 1) / U_ROWS); };
+  ISPA_CK(launch_pdl(col_exp_kernel<false>, col_grid(D), dim3(256), 0, s, gram + D, ldg, D, D,
+                     static_cast<const int32_t*>(w.t), -1, w.u));
+  ISPA_CK(launch_pdl(col_exp_kernel<true>, col_grid(d_out), dim3(256), 0, s, W, static_cast<int64_t>(d_out), D, d_out,
+                     static_cast<const int32_t*>(w.u), 1, w.ew));
 
   // tr(W^T S W) = sum_ij S_ij (W W^T)_ij: W's rows sliced over d_out
   ISPA_CK(slice_rows<float>(slice(W, d_out, D, d_out, w.kn, w.t_d, w.op_a, w.ea), Dp, 1, s));
@@ -576,9 +627,17 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     p.dot = w.scal + 2;
     ISPA_CK(launch_slice_gemm<SL_DOT>(p, sms, s));
   }
-  // B = 2^-t X W
-  ISPA_CK(slice_rows<float>(slice(gram + D, ldg, D, D, Dp, w.t_d, w.op_a, w.ea), Dp, 1, s));
-  ISPA_CK(slice_cols<float>(slice(W, d_out, d_out, D, Dp, w.t_n, w.op_b, w.eb), w.np, 1, s));
+  // B = 2^-t X W = 2^-t (X 2^-u) (2^u W)
+  {
+    SliceParams x = slice(gram + D, ldg, D, D, Dp, w.t_d, w.op_a, w.ea);
+    SliceParams y = slice(W, d_out, d_out, D, Dp, w.t_n, w.op_b, w.eb);
+    x.k_exp = y.k_exp = w.u;
+    x.k_sign = -1;
+    y.k_sign = 1;
+    y.r_max = w.ew;
+    ISPA_CK((slice_rows<float, SL_FULL, true>(x, Dp, 1, s)));
+    ISPA_CK((slice_cols<float, SL_FULL, true>(y, w.np, 1, s)));
+  }
   {
     SlGemm p = base;
     p.a = w.op_a;
