@@ -657,11 +657,20 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(const SlGemm 
     if constexpr (MODE == SL_DOT) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-      if (lane == 0) atomicAdd(p.dot, dot);
+      // the stages are free: a warp is done once all of this CTA's sums have been read
+      if (lane == 0) reinterpret_cast<double*>(smem)[warp - 2] = dot;
     }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (MODE == SL_DOT) {
+    // one addition a CTA: each rounds the whole sum, and one a warp cost eps as many bits as all else
+    if (threadIdx.x == 0) {
+      double sum = 0.0;
+      for (int i = 0; i < SG_EPI; ++i) sum += reinterpret_cast<const double*>(smem)[i];
+      atomicAdd(p.dot, sum);
+    }
+  }
   if (threadIdx.x == 0 && *abort_flag) atomicOr(p.flag, 2);
   if (warp == 1) {
     tc_fence_after();

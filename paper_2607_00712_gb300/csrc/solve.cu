@@ -461,24 +461,28 @@ __global__ void __launch_bounds__(256) sumsq_kernel(const double* __restrict__ x
   block_add(s, out);
 }
 
-// dW[i][j] = z[j][i] 2^(-t_i), through 32 x 32 tiles; *out += ||dW||^2 (before the fp32 rounding).
+// dW[i][j] = z[j][i] 2^(-t_i), through 32 x 32 tiles, a CTA every gridDim.y-th of its rows; *out += ||dW||^2 (before
+// the fp32 rounding).
 __global__ void __launch_bounds__(256) finish_kernel(const double* __restrict__ z, int D, int Dp, int n,
                                                      const int32_t* __restrict__ t, float* __restrict__ dW, double* out) {
   __shared__ float tile[32][33];
   pdl_wait();
   pdl_trigger();
-  const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+  const int i0 = blockIdx.x * 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   double s = 0.0;
-  for (int jj = w; jj < 32; jj += 8) {
-    double v = 0.0;
-    if (j0 + jj < n && i0 + lane < D) v = z[static_cast<int64_t>(j0 + jj) * Dp + i0 + lane] * pow2d(-t[i0 + lane]);
-    s = fma(v, v, s);
-    tile[jj][lane] = static_cast<float>(v);
+  for (int j0 = blockIdx.y * 32; j0 < n; j0 += gridDim.y * 32) {
+    for (int jj = w; jj < 32; jj += 8) {
+      double v = 0.0;
+      if (j0 + jj < n && i0 + lane < D) v = z[static_cast<int64_t>(j0 + jj) * Dp + i0 + lane] * pow2d(-t[i0 + lane]);
+      s = fma(v, v, s);
+      tile[jj][lane] = static_cast<float>(v);
+    }
+    __syncthreads();
+    for (int ii = w; ii < 32; ii += 8)
+      if (i0 + ii < D && j0 + lane < n) dW[static_cast<int64_t>(i0 + ii) * n + j0 + lane] = tile[lane][ii];
+    __syncthreads();
   }
-  __syncthreads();
-  for (int ii = w; ii < 32; ii += 8)
-    if (i0 + ii < D && j0 + lane < n) dW[static_cast<int64_t>(i0 + ii) * n + j0 + lane] = tile[lane][ii];
   block_add(s, out);
 }
 
@@ -767,7 +771,9 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     for (int k = k1 - 1; k >= z * (w.win / TB); --k) ISPA_CK(step(k, w.op_it, w.eit, z * w.win, k * TB));
     if (z > 0) ISPA_CK(far(z, 0, z * w.win));
   }
-  ISPA_CK(launch_pdl(finish_kernel, dim3((D + 31) / 32, (d_out + 31) / 32), dim3(256), 0, s,
+  // no more CTAs than fill the chip: each adds to the one sum
+  const unsigned fx = (D + 31) / 32, fy = (d_out + 31) / 32, fmax = fx < 8u * sms ? 8u * sms / fx : 1u;
+  ISPA_CK(launch_pdl(finish_kernel, dim3(fx, fy < fmax ? fy : fmax), dim3(256), 0, s,
                      static_cast<const double*>(w.B), D, Dp, d_out, static_cast<const int32_t*>(w.t), dW, w.scal + 1));
   struct {
     double scal[4];
