@@ -195,9 +195,11 @@ ISPA_API ispa_status ispa_debug_error_record(int32_t* rec8);
  * NULL / 0 turns it off (the default). */
 ISPA_API ispa_status ispa_debug_set_heartbeat(uint32_t* counters, int32_t n_slots);
 
-/* Debug aid: per-key-tile cycle trace of CTA (0, 0) of the bf16, head_dim 128
- * attention kernel (a separate instance of it, launched while a buffer is set;
- * it computes the same results).
+/* Debug aid: per-key-tile cycle trace of the first CTA of a bf16, head_dim 128
+ * attention call (a separate instance of its kernel, launched while a buffer is
+ * set; it computes the same results): the key tiles of its first work item.  Items
+ * that are split over clusters after whole ones leave no events; in a call whose
+ * items are all split, the first CTA records the tiles of its share.
  * buf: device-accessible uint64 [n_tiles][32], clock64 values, zero where an
  * event is not recorded.  The counters of an SM's four sub-partitions are not
  * aligned with one another: compare stamps of warps on different sub-partitions
@@ -210,7 +212,7 @@ ISPA_API ispa_status ispa_debug_set_heartbeat(uint32_t* counters, int32_t n_slot
  *   15 (j >= 1)        UMMA thread: K_j landed;
  *   6, 7               TMA thread: K_j issued, V_j issued;
  *   16 + w, 24 + w     softmax warp w (0-7): P_j arrived, S_j seen;
- *   12-15 of tile 0    once per CTA: kernel entry, TMEM allocated, Q tile landed,
+ *   12-15 of tile 0    once: kernel entry, TMEM allocated, Q tile landed,
  *                      epilogue stored.
  * NULL / 0 turns it off (the default). */
 ISPA_API ispa_status ispa_debug_set_trace(uint64_t* buf, int32_t n_tiles);
@@ -218,7 +220,8 @@ ISPA_API ispa_status ispa_debug_set_trace(uint64_t* buf, int32_t n_tiles);
 /* Debug aid for the timeout path: while tile >= 0, the TMA thread of every attention CTA
  * stops before loading key tile `tile` (it issues nothing more and drains what it issued),
  * so the UMMA thread's wait for that tile runs out after the wait limit and the CTA leaves
- * through its abort path, recording ISPA_ERR_TIMEOUT.  CTAs with fewer tiles run normally.
+ * through its abort path, recording ISPA_ERR_TIMEOUT.  CTAs with fewer tiles, and those of a split
+ * item whose share does not hold it, run normally.
  * Nothing faults: the missing load simply never arrives.  -1 turns it off (the default). */
 ISPA_API ispa_status ispa_debug_drop_k_tile(int32_t tile);
 

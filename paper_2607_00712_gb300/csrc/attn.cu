@@ -204,7 +204,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // rows over the cluster through distributed shared memory, the LSE fusion of Eq. 11-12.  No
 // workspace, no second launch, no dual mode.
 // TRACE: the instance launched while a trace buffer is set records the per-tile events of
-// ispa_debug_set_trace (first work item of CTA (0, 0)); the production instances contain no
+// ispa_debug_set_trace (first work item of the call's first CTA); the production instances contain no
 // trace code at all (even an untaken clock64 read constrains instruction scheduling: it cost 6 %
 // here).
 //
@@ -983,6 +983,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           p.lse[static_cast<size_t>(head) * p.n_q + qrow] = (m - C::P_SHIFT + __log2f(l)) * 0.69314718055994531f;
       }
     }
+    if (threadIdx.x == 0) tr(0, 15);   // epilogue stored
     cluster_sync();   // no CTA leaves while another still reads its shared memory
     if (!p.wait_first) pdl_wait();   // the launch of the whole items completes before this one does
   }
@@ -1087,6 +1088,7 @@ static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, cons
     if (e != cudaSuccess) return e;
     p.item0 = first;
     p.wait_first = first == 0;
+    if (first > 0) p.trace = nullptr;   // the events are those of the whole items' first CTA
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(plan.items * plan.c));
     cfg.blockDim = dim3(NTHREADS);

@@ -48,7 +48,7 @@ struct AttnParams {
   float* disc_part;        // [H][n_q] per-head sum of squared discrepancy (dual)
   int* status;             // library status record
   uint32_t* heartbeat;     // debug counters (host-mapped) or null
-  uint64_t* trace;         // debug per-tile cycle trace of CTA (0,0) or null: [tile][8]
+  uint64_t* trace;         // debug per-tile cycle trace of the first CTA or null: [tile][32]
   int32_t trace_tiles;
   int32_t drop_k_tile;     // debug: key tile the TMA thread never loads (-1: none)
   // 8-bit Q K^T (null for bf16 Q and K): per-head e4m3 code scales of q, chunk keys, ring keys
