@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + C::N_BAR);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  uint32_t* issued = tmem_slot + 2;   // PAIR: k-blocks loaded by this CTA's producer; the other CTA's word
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * QST, accf0 = empty0 + 8 * QST,
                  acce0 = accf0 + 16, drain_bar = acce0 + 16;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -295,13 +296,11 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
           }
         }
       }
-      if (rank == 0) {
+      if constexpr (PAIR) {
+        issued[0] = static_cast<uint32_t>(g);   // a pair drains at its end
+      } else {
         for (int i = g > QST ? g - QST : 0; i < g; ++i)
           mbar_wait_drain(full0 + 8 * (i % QST), (i / QST) & 1, Q_DRAIN_NS);
-      } else if (!ok) {
-        // after a timeout: rank 1's loads count on rank 0's barriers, so give those in flight time to land
-        const uint64_t t0 = globaltimer_ns();
-        while (globaltimer_ns() - t0 < 1000 * 1000) __nanosleep(1000);
       }
     }
     __syncwarp();
@@ -452,7 +451,28 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
     }
     cluster_sync();   // no CTA leaves while another still reads its shared memory
   }
-  if constexpr (PAIR) cluster_sync();   // neither CTA's TMEM, barriers or shared memory is used by the other any more
+  if constexpr (PAIR) {
+    // Without a timeout rank 0's UMMA thread has waited for every load.  After one the two producers may have
+    // stopped at different k-blocks, and rank 1's loads count on rank 0's barriers: the CTAs tell each other how far
+    // they got, rank 0 waits for what is in flight, and neither leaves before that.
+    constexpr uint32_t kAborted = 1u << 31;
+    const uint32_t mine = issued[0] | (*abort_flag ? kAborted : 0u);
+    if (threadIdx.x == 0) cluster_st1(cluster_map(smem_u32(issued + 1), rank ^ 1), mine);
+    cluster_sync();   // neither CTA's TMEM, barriers or shared memory is used by the other's roles any more
+    const uint32_t other = issued[1];
+    if ((mine | other) & kAborted) {
+      if (rank == 0 && threadIdx.x == 0) {
+        const int g0 = static_cast<int>(mine & ~kAborted), g1 = static_cast<int>(other & ~kAborted), g = max(g0, g1);
+        for (int i = max(g - QST, 0); i < g; ++i) {   // the last round of every stage
+          const uint32_t bar = full0 + 8 * (i % QST);
+          if (i >= g0) mbar_arrive_expect_tx(bar, C::STAGE);   // rank 1's half only
+          if (i >= g1) mbar_complete_tx(bar, C::STAGE);        // rank 1's half was never asked for
+          mbar_wait_drain(bar, (i / QST) & 1, Q_DRAIN_NS);
+        }
+      }
+      cluster_sync();
+    }
+  }
   if (warp == 1) {
     tc_fence_after();
     if constexpr (PAIR) tmem_dealloc_pair(tmem, C::TMEM_COLS);
