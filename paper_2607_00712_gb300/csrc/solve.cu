@@ -165,12 +165,38 @@ __device__ __forceinline__ void pivot_rsqrt(int64_t d, uint64_t& y, int& e) {
   y = (static_cast<uint64_t>(m) << 39) + static_cast<uint64_t>((static_cast<int64_t>(m) * corr) >> 21);
 }
 
-// c (62 fraction bits) times y 2^e with 63 fraction bits; a magnitude of 1 or more sets `over`.
-__device__ __forceinline__ int64_t scale_col(int64_t c, uint64_t y, int e, bool& over) {
+// An element of L as the panel's dot products take it: x 2^-30 + y 2^-58, rounded, y signed (28 bits).  A multiply-add
+// is then three 32 x 32 + 64 bit ones without any shift or carry (a 64-bit multiply-high takes 21 issue slots, these
+// 12); the middle sums of 64 products of rows whose norm is at most 1 stay below 2^62.  What is lost is half of 2^-58
+// of the other factor a term and the product of the two y, 2^-62 at most, both either way, where fp64 rounds the
+// running sum to 2^-54 of itself.  A square's y^2 is never negative: its mean goes into the rounding (a square of 0
+// stays 0).  With y cut off and unsigned the diagonal of L L^T was 6e-18 too large, and eps of ill-conditioned systems
+// 3e-14 of its terms off (here 2e-15, plain fp64 code 8e-15 to 4e-14); a fourth product for the two y gave the same
+// as this but 6 us a panel.
+__device__ __forceinline__ int2 pack_l(int64_t l) {   // 60 fraction bits
+  return make_int2(static_cast<int>((l + 2 + (1 << 29)) >> 30),
+                   static_cast<int>((static_cast<uint32_t>(l) + 2) << 2) >> 4);
+}
+struct Dot {
+  int64_t hi = 0, mid = 0;
+  __device__ __forceinline__ void add(const int2 a, const int2 b) {
+    hi += static_cast<int64_t>(a.x) * b.x;
+    mid += static_cast<int64_t>(a.x) * b.y;
+    mid += static_cast<int64_t>(a.y) * b.x;
+  }
+  // 62 fraction bits
+  __device__ __forceinline__ int64_t sum(int round = 1 << 25) const { return (hi << 2) + ((mid + round) >> 26); }
+  __device__ __forceinline__ int64_t square() const { return sum((1 << 25) + (1 << 26) / 3); }
+};
+
+// c (62 fraction bits) times y 2^e with 63 fraction bits; a magnitude of 1 or more sets `over`.  pk: the same for the
+// dot products.
+__device__ __forceinline__ int64_t scale_col(int64_t c, uint64_t y, int e, bool& over, int2& pk) {
   const int64_t c1 = static_cast<int64_t>(static_cast<uint64_t>(c) << (e + 1));
   const __int128 p = static_cast<__int128>(c1) * static_cast<int64_t>(y >> 1);
-  const int64_t hi = static_cast<int64_t>(p >> 64);
+  const int64_t hi = static_cast<int64_t>(p >> 64);   // 60 fraction bits
   over |= (c1 >> (e + 1)) != c || static_cast<uint64_t>(hi + (int64_t{1} << 60)) >= (uint64_t{1} << 61);
+  pk = pack_l(hi);
   return static_cast<int64_t>(p >> 61);
 }
 
@@ -184,24 +210,6 @@ struct PanelParams {
   int* flag;
   int* status;
   uint64_t wait_limit_ns;
-};
-
-// Elements of L as the panel's dot products take them: the high word of the 63 fraction bits and the
-// next 27 bits.  A multiply-add is then three 32 x 32 + 64 bit ones without any shift or carry (a 64-bit
-// multiply-high takes 21 issue slots, these 12); the middle sums of 64 products of rows whose norm is at most 1
-// stay below 2^63.  What is dropped is below 2^-58 of the other factor a term, where fp64 rounds the
-// running sum to 2^-54 of itself.
-__device__ __forceinline__ int2 pack_l(int64_t l) {
-  return make_int2(static_cast<int>(l >> 32), static_cast<int>(static_cast<uint32_t>(l) >> 5));
-}
-struct Dot {
-  int64_t hi = 0, mid = 0;
-  __device__ __forceinline__ void add(const int2 a, const int2 b) {
-    hi += static_cast<int64_t>(a.x) * b.x;
-    mid += static_cast<int64_t>(a.x) * b.y;
-    mid += static_cast<int64_t>(a.y) * b.x;
-  }
-  __device__ __forceinline__ int64_t sum() const { return hi + (mid >> 27); }   // 62 fraction bits
 };
 
 // One panel: every CTA factors the 64 x 64 diagonal block for itself (the same work on every SM, and
@@ -299,9 +307,7 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
     for (int j = 0; j < NB; ++j) {
       chain_sync();   // pivot j
       if (r > j) {
-        const int64_t l = scale_col(cs[r], ys[j], es[j], over);
-        pk[r * PLD + j] = pack_l(l);
-        a[r * PLD + j] = l;
+        a[r * PLD + j] = scale_col(cs[r], ys[j], es[j], over, pk[r * PLD + j]);
       }
       chain_sync();   // column j
     }
@@ -314,8 +320,8 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
         const int2 l0 = pk[lane * PLD + j - 1], l1 = pk[(lane + 32) * PLD + j - 1];
         q0.add(l0, l0);
         q1.add(l1, l1);
-        d0 -= lane >= j ? q0.sum() : 0;
-        d1 -= lane + 32 >= j ? q1.sum() : 0;
+        d0 -= lane >= j ? q0.square() : 0;
+        d1 -= lane + 32 >= j ? q1.square() : 0;
       }
       int64_t d = __shfl_sync(0xffffffffu, j < 32 ? d0 : d1, j & 31);
       if (d <= 0) {
@@ -349,10 +355,11 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
       int64_t sum = acc.sum();
 #pragma unroll
       for (int o = PL / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      const int64_t l = scale_col(a[r * PLD + j] - sum, ys[j], es[j], over);
+      int2 packed;
+      const int64_t l = scale_col(a[r * PLD + j] - sum, ys[j], es[j], over, packed);
       __syncwarp();
       if (h == 0) {
-        row[j] = pack_l(l);
+        row[j] = packed;
         a[r * PLD + j] = l;
       }
       __syncwarp();

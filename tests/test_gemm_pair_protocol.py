@@ -1,13 +1,13 @@
 """A model of the barrier schedule of the W8A8 GEMM's pairs of CTAs (csrc/w8a8.cu, cta_group::2), checked over every
 interleaving, with and without a wait that runs out.
 
-Both producers wait for their own empty barriers (one commit of rank 0's UMMA thread arrives at both) and load their half
-of a k-block; both halves count on rank 0's full barrier of the stage, which rank 0's producer arms for both. The
+Both producers wait for their own empty barriers (one commit of rank 0's UMMA thread arrives at both) and load their
+half of a k-block; both halves count on rank 0's full barrier of the stage, which rank 0's producer arms for both. The
 UMMA thread of rank 0 waits for the full barriers and for the accumulator set (an arrival from either CTA's read-back
-warps), and commits the set to both. A role whose wait runs out, or whose CTA has aborted, stops there. At the end the CTAs
-exchange how many k-blocks their producers have loaded and whether they have aborted; if either has, rank 0 goes
-through the last round of every stage: it arms what it has not armed, takes back what rank 1 has not loaded, and waits for
-the rest.
+warps), and commits the set to both. A role whose wait runs out, or whose CTA has aborted, stops there. At the end the
+CTAs exchange how many k-blocks their producers have loaded and whether they have aborted; if either has, rank 0 goes
+through the last round of every stage: it arms what it has not armed, takes back what rank 1 has not loaded, and waits
+for the rest.
 
 Checked: a stage is loaded again only after the UMMAs that read it, an accumulator set is written only after both CTAs
 have read it, every run ends, and no load is in flight when the CTAs leave."""
