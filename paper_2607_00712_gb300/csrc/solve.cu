@@ -576,10 +576,10 @@ cudaError_t slice_rows(const SliceParams& p, int grid_rows, int n_seg, cudaStrea
 }
 
 template <typename T, int TRI = SL_FULL, bool SCALED = false>
-cudaError_t slice_cols(const SliceParams& p, int grid_rows, int n_seg, cudaStream_t s) {
+cudaError_t slice_cols(const SliceParams& p, int grid_rows, int n_seg, int sms, cudaStream_t s) {
   dim3 grid((grid_rows + 31) / 32, n_seg);
   const int warps = p.k_pad > 128 ? 32 : 8, most = p.k_pad / 8 / warps;   // parts with work for every warp
-  const int fill = 304 / static_cast<int>(grid.x * grid.y);
+  const int fill = 2 * sms / static_cast<int>(grid.x * grid.y);
   grid.z = fill < 1 || most < 1 ? 1 : (fill < most ? fill : most);
   return launch_pdl(slice_cols_kernel<T, TRI, SCALED>, grid, dim3(32 * warps), 0, s, p);
 }
@@ -625,11 +625,10 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     p.a = p.b = w.op_a;
     p.a_chunk = p.b_chunk = chunk_d;
     p.ea = p.eb = w.ea;
-    // the sum over the contraction index too can be cut: as many pieces of at least two flushes
-    // as make the last wave's idle SMs a small part of the whole
-    const int mt = Dp / 128, chunks = w.kn / SL_K;
-    p.n_split = chunks / (2 * SG_FLUSH) < 1 ? 1 : (chunks / (2 * SG_FLUSH) > 8 ? 8 : chunks / (2 * SG_FLUSH));
-    while (p.n_split > 1 && mt * (mt + 1) > 8 * sms) --p.n_split;
+    // the sum over the contraction index too can be cut, into up to eight pieces of at least two flushes; with eight
+    // waves of tiles the last one's idle SMs are a small part of the whole anyway
+    const int mt = Dp / 128, chunks = w.kn / SL_K, pieces = chunks / (2 * SG_FLUSH);
+    p.n_split = pieces < 1 || mt * (mt + 1) > 8 * sms ? 1 : (pieces > 8 ? 8 : pieces);
     p.n_tiles = mt * (mt + 1) * p.n_split;
     p.n_chunks = chunks;
     p.row_end = D;
@@ -647,7 +646,7 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     y.k_sign = 1;
     y.r_max = w.ew;
     ISPA_CK((slice_rows<float, SL_FULL, true>(x, Dp, 1, s)));
-    ISPA_CK((slice_cols<float, SL_FULL, true>(y, w.np, 1, s)));
+    ISPA_CK((slice_cols<float, SL_FULL, true>(y, w.np, 1, sms, s)));
   }
   {
     SlGemm p = base;
@@ -701,7 +700,7 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
     ISPA_CK((slice_rows<double, SL_LOWER>(q, TB, nb, s)));
     q.op = w.op_it;
     q.exps = w.eit;
-    ISPA_CK((slice_cols<double, SL_UPPER>(q, TB, nb, s)));
+    ISPA_CK((slice_cols<double, SL_UPPER>(q, TB, nb, sms, s)));
   }
 
   // B's rows [r0, r0 + n) sliced, over all columns
@@ -757,8 +756,8 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
   near_l.lower = far_l.lower = 1;
   near_l.z_src = TB * ld;
   far_l.z_src = w.win * ld;
-  if (nb > 1) ISPA_CK(slice_cols<int64_t>(near_l, w.win, nb, s));
-  if (n_win > 1) ISPA_CK(slice_cols<int64_t>(far_l, Dp, n_win - 1, s));
+  if (nb > 1) ISPA_CK(slice_cols<int64_t>(near_l, w.win, nb, sms, s));
+  if (n_win > 1) ISPA_CK(slice_cols<int64_t>(far_l, Dp, n_win - 1, sms, s));
   for (int z = 0; z < n_win; ++z) {
     const int k1 = (z + 1) * (w.win / TB) < nb ? (z + 1) * (w.win / TB) : nb;
     for (int k = z * (w.win / TB); k < k1; ++k) ISPA_CK(step(k, w.op_i, w.ei, (k + 1) * TB, k1 * TB));
