@@ -1080,7 +1080,8 @@ static cudaError_t launch_hd(const CUtensorMap* tq, const CUtensorMap* tkr, cons
   p.item0 = 0;
   p.wait_first = 1;
   if (first > 0) {
-    e = launch_pdl(whole, dim3(static_cast<unsigned>(first)), dim3(NTHREADS), C::SMEM, s, *tq, *tkr, *tvr, *tkc, *tvc, p);
+    e = launch_pdl(whole, dim3(static_cast<unsigned>(first)), dim3(NTHREADS), C::SMEM, s, *tq, *tkr, *tvr, *tkc, *tvc,
+                   p);
     if (e != cudaSuccess) return e;
   }
   if (plan.items > 0) {

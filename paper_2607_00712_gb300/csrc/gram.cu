@@ -793,8 +793,8 @@ __global__ void __launch_bounds__(W_THREADS, 1)
 // with m CTAs for every pass each works on one tile; with one CTA per SM most CTAs get the end of one tile and
 // the beginning of another, a second read-back and flush worth `flush` steps.  Of the two the
 // one whose CTAs finish first, by a fit to measured runs (steps take 5 % longer on m CTAs a pass, whose flushes
-// come all at once).  Fewer CTAs than either never pay: a call of few tokens is bound by the read-backs and flushes that
-// a CTA does one after another, 5 us each for a 256 x 256 tile.  Before (16 steps or more for every CTA) and after, us:
+// come all at once).  Fewer CTAs than either never pay: a call of few tokens is bound by the read-backs and flushes
+// that a CTA does one after another, 5 us each for a 256 x 256 tile.  Before (16 steps or more a CTA) and after, us:
 // D 1536 with 60 tokens 97 -> 13.0, 300 tokens 36 -> 15.8; D 512 with 1000 tokens 21.4 -> 14.9, 4680 tokens
 // 30.9 -> 21.9; D 2048 with 2000 tokens 42.6 -> 38.8; D 384 with 1000 tokens 15.2 -> 10.0.
 static int gram_grid(int64_t total, int64_t len, int sms, int flush) {

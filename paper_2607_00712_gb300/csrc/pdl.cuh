@@ -2,8 +2,9 @@
 // kernel launched with launch_pdl may start (and run its prologue: barrier set-up, TMEM
 // allocation) while the kernel before it finishes; it calls pdl_wait() before its first
 // access to global memory that the earlier kernel may write (or, for a write of its own, may
-// still read), which returns once that kernel has completed and its writes are visible.  pdl_trigger() in the earlier kernel lets the
-// dependent start before all of its blocks have exited.
+// still read), which returns once that kernel has completed and its writes are visible.
+// pdl_trigger() in the earlier kernel lets the dependent start before all of its blocks have
+// exited.
 #pragma once
 
 #include <cuda_runtime.h>

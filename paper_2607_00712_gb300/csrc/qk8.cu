@@ -193,7 +193,8 @@ struct QuantVtParams {
   int32_t slot[kMaxAppendFrames];
 };
 
-__device__ __forceinline__ void quant_vt_block(const QuantVtParams& p, int64_t t0, int h, uint32_t (*tile)[VT_TOK / 4]) {
+__device__ __forceinline__ void quant_vt_block(const QuantVtParams& p, int64_t t0, int h,
+                                               uint32_t (*tile)[VT_TOK / 4]) {
   const int rows = static_cast<int>(p.n - t0 < VT_TOK ? p.n - t0 : VT_TOK);
   const int c8 = threadIdx.x & 15;
   uint4 x[2][4];
@@ -215,7 +216,8 @@ __device__ __forceinline__ void quant_vt_block(const QuantVtParams& p, int64_t t
     for (int r = 0; r < 4; ++r) q[r] = quant8(x[i][r], inv);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {   // 4 x 4 bytes: tokens x channels -> channels x tokens
-      const uint32_t a0 = k ? q[0].y : q[0].x, a1 = k ? q[1].y : q[1].x, a2 = k ? q[2].y : q[2].x, a3 = k ? q[3].y : q[3].x;
+      const uint32_t a0 = k ? q[0].y : q[0].x, a1 = k ? q[1].y : q[1].x;
+      const uint32_t a2 = k ? q[2].y : q[2].x, a3 = k ? q[3].y : q[3].x;
       const uint32_t l0 = __byte_perm(a0, a1, 0x5140), l1 = __byte_perm(a2, a3, 0x5140);
       const uint32_t h0 = __byte_perm(a0, a1, 0x7362), h1 = __byte_perm(a2, a3, 0x7362);
       uint32_t* row = &tile[8 * c8 + 4 * k][t4 ^ (2 * c8)];
@@ -382,8 +384,8 @@ cudaError_t launch_quant_q_blocks(const void* x, int64_t n, int32_t H, int32_t d
                                   cudaStream_t s) {
   const dim3 grid(static_cast<unsigned>((n + QB - 1) / QB), static_cast<unsigned>(H));
   return launch_pdl(d <= 128 ? quant_q_blocks_kernel<8> : quant_q_blocks_kernel<16>, grid, dim3(256), 0, s,
-                    static_cast<const uint4*>(x), n, static_cast<int>(H), static_cast<int>(d), reinterpret_cast<uint2*>(q),
-                    scale);
+                    static_cast<const uint4*>(x), n, static_cast<int>(H), static_cast<int>(d),
+                    reinterpret_cast<uint2*>(q), scale);
 }
 
 cudaError_t launch_quant_given(const void* x, int64_t n, int32_t H, int32_t d, const float* scale, uint8_t* q,

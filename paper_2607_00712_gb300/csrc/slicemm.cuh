@@ -5,9 +5,9 @@
 //   x ~= 2^E * sum_p d_p 2^(-7-8p),
 // what is left over being below 2^-56 of the row's largest magnitude (E is the row's own power of
 // two).  A product of two such rows is sum_s 2^(-14-8s) v_s with v_s = sum_{p+q=s} <d_p, d'_q>, s = 0 .. 7
-// (the pairs beyond weigh less than the digits' own remainder; without s = 7 the solve's error, 6e-16 to
-// 2e-15 against 64-bit arithmetic's 5e-16 to 1e-15 on well-conditioned systems, was up to twice as large).  Digits are bf16 numbers,
-// their products integers up to 2^14, and over 128 products of at most 7 pairs a v_s stays below
+// (the pairs beyond weigh less than the digits' own remainder; without s = 7 the solve's error on
+// well-conditioned systems, 3e-16 of dW against 1e-15 in fp64 arithmetic, was up to twice as large).  Digits are bf16
+// numbers, their products integers up to 2^14, and over 128 products of at most 7 pairs a v_s stays below
 // 2^24: the fp32 accumulators of the tensor cores hold it exactly.  So every 128 products the
 // accumulators are read back and added up as 64-bit integers, and a whole contraction is exact
 // but for the digits dropped, in a fixed-point word of 2^-70 of the two rows' scales.  This is the
@@ -98,7 +98,8 @@ __device__ __forceinline__ int64_t sl_offset(int64_t chunk, int n_t, int r, int 
 // A number is rounded to 56 bits; with 128 added at every digit but the first its bytes are the digits plus 128
 // (the first keeps its sign and range [-128, 128]), so that a digit costs a byte permute and an addition: byte b under
 // the exponent of 2^23 is the fp32 number 2^23 + b.  Rounding and subtracting 64-bit digits one after another took five
-// times as many instructions: with fixed_to_double's funnel shifts a 1536 x 1536 solve 3.07 -> 2.93 ms, 5120 x 5120 28.4 -> 27.5.
+// times as many instructions: with fixed_to_double's funnel shifts a 1536 x 1536 solve went from 3.07 to 2.93 ms,
+// 5120 x 5120 from 28.4 to 27.5.
 __device__ __forceinline__ void store_digits8(const int64_t* xi, uint8_t* dst) {
   constexpr float kBias = 8388608.f + 128.f;
   uint32_t lo[8], hi[8];
@@ -362,8 +363,8 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 }
 
 // (hi 2^32 + lo) 2^e rounded to nearest, without the fp64 pipe (2 operations per clock and SM); e is a row's and a
-// column's exponent and a few tens: normal results only need the integer path, in 32-bit words and funnel shifts, the rest goes
-// through ldexp.
+// column's exponent and a few tens: normal results only need the integer path, in 32-bit words and funnel shifts, the
+// rest goes through ldexp.
 __device__ __forceinline__ double fixed_to_double(int64_t hi, uint32_t lo, int e) {
   const uint32_t sign = static_cast<uint32_t>(static_cast<uint64_t>(hi) >> 32) & 0x80000000u;
   const uint32_t neg = static_cast<uint32_t>(static_cast<int32_t>(sign) >> 31);   // all ones for a negative number
@@ -390,8 +391,8 @@ __device__ __forceinline__ double fixed_to_double(int64_t hi, uint32_t lo, int e
   // 53 bits; a carry out raises the exponent by itself
   const uint64_t m = (static_cast<uint64_t>(m1 >> 11) << 32 | __funnelshift_r(m0, m1, 11)) + ((m0 >> 10) & 1);
   if (ex < 1 || ex > 2045) return ldexp(sign ? -static_cast<double>(m) : static_cast<double>(m), ex - 1023 - 52);
-  return __hiloint2double(static_cast<int>((static_cast<uint32_t>(ex - 1) << 20) + static_cast<uint32_t>(m >> 32) + sign),
-                          static_cast<int>(static_cast<uint32_t>(m)));
+  const uint32_t top = (static_cast<uint32_t>(ex - 1) << 20) + static_cast<uint32_t>(m >> 32) + sign;
+  return __hiloint2double(static_cast<int>(top), static_cast<int>(static_cast<uint32_t>(m)));
 }
 
 __device__ __forceinline__ double pow2d(int e) {   // 2^e; 0 below the normal range, inf above it
@@ -470,7 +471,8 @@ __device__ __forceinline__ bool sg_read_sums(int64_t (&hi)[SG_COLS], uint32_t (&
         const int u0 = __float2int_rn(__uint_as_float(v[0][i])), u1 = __float2int_rn(__uint_as_float(v[1][i]));
         const int u2 = ns > 2 ? __float2int_rn(__uint_as_float(v[2][i])) : 0;
         if (h == 0) {
-          hi[8 * c + i] += static_cast<int64_t>(u0 * 256 + u1) * 65536 + static_cast<int64_t>(u2) * 256;   // |u0| <= 2^21
+          // |u0| <= 2^21
+          hi[8 * c + i] += static_cast<int64_t>(u0 * 256 + u1) * 65536 + static_cast<int64_t>(u2) * 256;
         } else {
           if (h == 1) hi[8 * c + i] += u0;
           const int64_t l = h == 1 ? static_cast<int64_t>(u1) * (1 << 24)
@@ -611,7 +613,8 @@ __global__ void __launch_bounds__(SG_THREADS, 1) slice_gemm_kernel(const SlGemm 
 #pragma unroll
           for (int i = 0; i < SG_COLS; ++i) {
             const int sh = 8 - (ea + p.eb[min(col + i, row)]);   // exponents of factor rows are never above 0
-            hi[i] = sh <= 32 ? static_cast<int64_t>(static_cast<uint64_t>(hi[i]) << (32 - sh)) + (lo[i] >> min(sh, 31) >> (sh == 32))
+            const uint32_t rest = lo[i] >> min(sh, 31) >> (sh == 32);
+            hi[i] = sh <= 32 ? static_cast<int64_t>(static_cast<uint64_t>(hi[i]) << (32 - sh)) + rest
                              : hi[i] >> min(sh - 32, 63);
           }
           int64_t o[SG_COLS];   // all in flight at once; nothing above the diagonal

@@ -14,11 +14,13 @@
 // products with the inverses of L's 128 x 128 diagonal blocks, and tr(W^T S W) = sum_ij S_ij (W W^T)_ij, half
 // the work of S W and nothing to store.  Plain fp64 code ran all of it at 1.09 TFLOP/s, the chip's
 // fp64 rate: 782 ms at hidden 5120 and 33 ms at 1536 (where the panels' launches and latency counted
-// too), against 27.5 and 2.90 ms.  What bounds it now: at 5120 the products' tensor time and read-back (21
-// of 27 ms), at 1536 the chain of 24 panels (44 us each) and 24 block steps, one after another.
-// dW's error against 80-bit arithmetic, before its rounding to fp32, was 0.03 to 0.9 times the plain code's (dim 384,
-// five draws each): features of one size or spread by exp(2 N(0, 1)) 0.3 to 0.4, rank-deficient sums 0.6, rank 20 plus
-// noise 0.14, near-duplicate pairs 0.26, singular values falling to 1e-4 0.9; scaled condition numbers 13 to 3e7.
+// too), against 27.7 and 2.94 ms.  What bounds it now: at 5120 the products' tensor time and read-back (21
+// of 28 ms), at 1536 the chain of 24 panels (45 us each) and 24 block steps, one after another.
+// dW's error against 80-bit arithmetic, read before its rounding to fp32, at dim 384 (plain fp64 code's in brackets):
+// features of one size or spread by exp(2 N(0, 1)) 3e-16 (1e-15); sums of half as many tokens as features 6e-11
+// (1.2e-10), near-duplicate pairs 9e-11 (3.4e-10), rank 20 plus 1 % noise 2.4e-11 (3.5e-10), singular values falling to
+// 1e-4 1.3e-12 (1.5e-11).  Errors are relative to the largest rows of the scaled solution: a row 1e-6 of them, of
+// features that share no token with theirs, had 6e-11 of itself, where fp64 code had 7e-16.
 //
 // The factorisation runs in fixed point.  Row and column i are scaled by a power of two (exactly)
 // so that M_ii lies in [1/4, 1); then every |M_ij|, every element of every Schur complement and
@@ -115,7 +117,8 @@ __global__ void __launch_bounds__(256) col_exp_kernel(const float* __restrict__ 
 // fix[j][i] (i >= j) = M_ij 2^(-t_i - t_j) with 62 fraction bits, from G's upper triangle (row j of G is column
 // j here); the padding is the identity / 2.
 __global__ void __launch_bounds__(256) form_kernel(const float* __restrict__ gram, int D, int Dp, double lambda,
-                                                   const int32_t* __restrict__ t, int64_t* __restrict__ fix, int* flag) {
+                                                   const int32_t* __restrict__ t, int64_t* __restrict__ fix,
+                                                   int* flag) {
   pdl_wait();
   pdl_trigger();
   const int j = blockIdx.x;
@@ -237,7 +240,7 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
   int2* pk = reinterpret_cast<int2*>(psm + PROWS * PLD);           // L for the dot products
   uint64_t* ys = reinterpret_cast<uint64_t*>(psm + 2 * PROWS * PLD);   // the pivots' reciprocal roots
   int64_t* cs = reinterpret_cast<int64_t*>(ys + NB);               // column j before its scaling
-  uint64_t* done = reinterpret_cast<uint64_t*>(cs + NB);           // mbarrier j: column j of the diagonal block is complete
+  uint64_t* done = reinterpret_cast<uint64_t*>(cs + NB);           // mbarrier j: column j of the block is complete
   int* es = reinterpret_cast<int*>(done + NB);
   volatile int* abort_flag = es + NB;
   pdl_wait();
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
     const int64_t* row = a + (NB + lane) * PLD;
     uint64_t mx = 0;
 #pragma unroll 16
-    for (int k = 0; k < NB; ++k) mx |= static_cast<uint64_t>(SliceSrc<int64_t>::mag(row[k]));   // same leading bit as the maximum
+    for (int k = 0; k < NB; ++k) mx |= static_cast<uint64_t>(SliceSrc<int64_t>::mag(row[k]));   // top bit of the max
     const int E = SliceSrc<int64_t>::exp_of(mx);
     if (kc == 0) p.exps[r0 + lane] = E;
     int64_t xi[8];
@@ -394,8 +397,8 @@ __global__ void __launch_bounds__(P_THREADS) panel_kernel(const PanelParams p) {
 // Inverse I of L's 128 x 128 diagonal blocks, fp64.  The factor is stored by columns and leaves the other half of
 // its array free: I_ij goes to [i][j], where column i has no L (the 64 x 64 blocks on the diagonal are
 // L's in `diag`).  One CTA per 8 columns of a block; thread (column, row group): right-looking substitution with its
-// rows in registers.  The CTAs of all blocks' first columns, which have the longest chains, come first, and load only what they need: 117 -> 62 us at
-// 1536, 257 -> 151 at 5120.
+// rows in registers.  The CTAs of all blocks' first columns, which have the longest chains, come first, and load only
+// what they need: 117 -> 62 us at 1536, 257 -> 151 at 5120.
 constexpr int IC = 8;
 constexpr int IG = 256 / IC;   // row groups
 constexpr int INV_SMEM = (TB * (TB + 1) + 2 * IC + TB) * 8;
@@ -463,15 +466,16 @@ __global__ void __launch_bounds__(256) sumsq_kernel(const double* __restrict__ x
   pdl_wait();
   pdl_trigger();
   double s = 0.0;
-  for (int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; e < n; e += static_cast<int64_t>(gridDim.x) * 256)
-    s = fma(x[e], x[e], s);
+  const int64_t step = static_cast<int64_t>(gridDim.x) * 256;
+  for (int64_t e = static_cast<int64_t>(blockIdx.x) * 256 + threadIdx.x; e < n; e += step) s = fma(x[e], x[e], s);
   block_add(s, out);
 }
 
 // dW[i][j] = z[j][i] 2^(-t_i), through 32 x 32 tiles, a CTA every gridDim.y-th of its rows; *out += ||dW||^2 (before
 // the fp32 rounding).
 __global__ void __launch_bounds__(256) finish_kernel(const double* __restrict__ z, int D, int Dp, int n,
-                                                     const int32_t* __restrict__ t, float* __restrict__ dW, double* out) {
+                                                     const int32_t* __restrict__ t, float* __restrict__ dW,
+                                                     double* out) {
   __shared__ float tile[32][33];
   pdl_wait();
   pdl_trigger();
@@ -524,7 +528,8 @@ SolveWs carve(void* ws, int D, int d_out) {
     p += align256(bytes);
     return r;
   };
-  const size_t Dp = w.Dp, chunk_d = static_cast<size_t>(w.t_d) * SL_TILE, chunk_n = static_cast<size_t>(w.t_n) * SL_TILE;
+  const size_t Dp = w.Dp, chunk_d = static_cast<size_t>(w.t_d) * SL_TILE;
+  const size_t chunk_n = static_cast<size_t>(w.t_n) * SL_TILE;
   const size_t ka = Dp > static_cast<size_t>(w.kn) ? Dp : w.kn;
   w.op_a = take(ka / SL_K * chunk_d);
   const size_t opb = Dp / SL_K * chunk_n, fix = Dp * Dp * 8;
@@ -747,7 +752,8 @@ ispa_status run_ls_solve(int32_t D, const float* gram, const float* W, int32_t d
   };
   // L's values for both: blocks of 128 columns (forward; rows: backward) within the windows, the window's width outside
   const int n_win = (Dp + w.win - 1) / w.win;
-  SliceParams near_l = slice(w.fix, ld, Dp, TB, TB, w.t_d, w.op_n, w.en), far_l = slice(w.fix, ld, Dp, w.win, w.win, w.t_d, w.op_a, w.ea);
+  SliceParams near_l = slice(w.fix, ld, Dp, TB, TB, w.t_d, w.op_n, w.en);
+  SliceParams far_l = slice(w.fix, ld, Dp, w.win, w.win, w.t_d, w.op_a, w.ea);
   near_l.rows_total = far_l.ks_total = Dp;
   near_l.z_k = TB;
   near_l.win = far_l.z_k = w.win;

@@ -51,9 +51,9 @@ __device__ __forceinline__ uint16_t e4m3x2(float x0, float x1) {
 // 16-byte words (8 bf16 each) stay in registers between the max and the quantisation pass;
 // of longer rows the rest is read twice.
 template <int CACHE>
-__global__ void __launch_bounds__(256, CACHE <= 4 ? 5 : CACHE <= 6 ? 4 : CACHE <= 8 ? 3 : 2) quant_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows,
-                                                         int cols, uint8_t* __restrict__ q,
-                                                         float* __restrict__ scale) {
+__global__ void __launch_bounds__(256, CACHE <= 4 ? 5 : CACHE <= 6 ? 4 : CACHE <= 8 ? 3 : 2)
+    quant_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int cols, uint8_t* __restrict__ q,
+                      float* __restrict__ scale) {
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x & 31;
@@ -411,7 +411,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
                                 __fmul_rn(__fmul_rn(s1, sa), __shfl_sync(0xffffffffu, sw[c], 8 * q + 2 * e + 1)));
           }
           // 64-byte swizzle: 16-byte word q of row r at word q ^ (r / 2 mod 4)
-          *reinterpret_cast<uint4*>(b + lane * 64 + (q ^ ((lane >> 1) & 3)) * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+          *reinterpret_cast<uint4*>(b + lane * 64 + (q ^ ((lane >> 1) & 3)) * 16) =
+              make_uint4(pk[0], pk[1], pk[2], pk[3]);
         }
         fence_proxy_async_smem();
         __syncwarp();
@@ -481,14 +482,15 @@ __global__ void __launch_bounds__(Q_THREADS, 1)
 }
 
 template <int BN, bool PAIR, bool SPLIT = false>
-cudaError_t launch_gemm_bn(int split, const uint8_t* a_q, const float* a_scale, const uint8_t* w_q, const float* w_scale,
-                           int32_t T, int32_t D, int32_t Dout, __nv_bfloat16* out, int* status,
+cudaError_t launch_gemm_bn(int split, const uint8_t* a_q, const float* a_scale, const uint8_t* w_q,
+                           const float* w_scale, int32_t T, int32_t D, int32_t Dout, __nv_bfloat16* out, int* status,
                            uint64_t wait_limit_ns, cudaStream_t s) {
   using C = QCfg<BN, PAIR>;
   int dev = 0;
   cudaGetDevice(&dev);
   {
-    const cudaError_t e = set_smem_limit_once(reinterpret_cast<const void*>(w8a8_gemm_kernel<BN, PAIR, SPLIT>), C::SMEM);
+    const cudaError_t e =
+        set_smem_limit_once(reinterpret_cast<const void*>(w8a8_gemm_kernel<BN, PAIR, SPLIT>), C::SMEM);
     if (e != cudaSuccess) return e;
   }
   CUtensorMap ta, tw, to;
@@ -511,7 +513,8 @@ cudaError_t launch_gemm_bn(int split, const uint8_t* a_q, const float* a_scale, 
   int dev_sms = 152;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev);
   const int ctas = SPLIT ? split : C::CTAS, units = SPLIT ? p.n_tiles : std::min(p.n_tiles, dev_sms / ctas);
-  return launch_pdl_cluster(w8a8_gemm_kernel<BN, PAIR, SPLIT>, dim3(units * ctas), dim3(Q_THREADS), C::SMEM, ctas, s, ta, tw, to, p);
+  return launch_pdl_cluster(w8a8_gemm_kernel<BN, PAIR, SPLIT>, dim3(units * ctas), dim3(Q_THREADS), C::SMEM, ctas, s,
+                            ta, tw, to, p);
 }
 
 }  // namespace
@@ -523,11 +526,13 @@ cudaError_t launch_quant_rows(const void* x, int64_t rows, int32_t cols, uint8_t
   const int64_t want = (rows + 7) / 8;   // one warp per row, 8 warps per block
   const int64_t blocks = want < static_cast<int64_t>(sms) * 16 ? want : static_cast<int64_t>(sms) * 16;
   // No more registers than the row needs: latency bounds this kernel, and with fewer of them all rows are in flight
-  // at once.  4680 x 1536: 4.4 -> 3.2 us, 9400 x 1024: 7.0 -> 4.0 (against 12 words a lane for every row).  Rows of more than
-  // 3072 values keep 12 and read the rest twice: with 20 only 8 warps a SM fit, 8.1 -> 10.2 us at 5120.
+  // at once.  4680 x 1536: 4.4 -> 3.2 us, 9400 x 1024: 7.0 -> 4.0 (against 12 words a lane for every row).  Rows of
+  // more than 3072 values keep 12 and read the rest twice: with 20 only 8 warps a SM fit, 8.1 -> 10.2 us at 5120.
   const int words = (cols / 8 + 31) / 32;
-  const auto kernel = words <= 4 ? quant_rows_kernel<4> : words <= 6 ? quant_rows_kernel<6> : words <= 8 ? quant_rows_kernel<8>
-                                                                                      : quant_rows_kernel<12>;
+  const auto kernel = words <= 4   ? quant_rows_kernel<4>
+                      : words <= 6 ? quant_rows_kernel<6>
+                      : words <= 8 ? quant_rows_kernel<8>
+                                   : quant_rows_kernel<12>;
   return launch_pdl(kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, s,
                     static_cast<const __nv_bfloat16*>(x), rows, static_cast<int>(cols), q, scale);
 }
@@ -557,7 +562,8 @@ cudaError_t launch_w8a8_gemm(const uint8_t* a_q, const float* a_scale, const uin
   struct Shape {
     int bn, ctas, kblock_ns, start_ns;
   };
-  static constexpr Shape kShapes[4] = {{256, 2, 325, 4800}, {256, 1, 366, 3000}, {192, 1, 325, 3000}, {128, 1, 308, 3000}};
+  static constexpr Shape kShapes[4] = {
+      {256, 2, 325, 4800}, {256, 1, 366, 3000}, {192, 1, 325, 3000}, {128, 1, 308, 3000}};
   const int64_t m_tiles = (static_cast<int64_t>(T) + QM - 1) / QM;
   int best = -1;
   int64_t best_cost = 0;
@@ -572,10 +578,11 @@ cudaError_t launch_w8a8_gemm(const uint8_t* a_q, const float* a_scale, const uin
       best_cost = cost;
     }
   }
-  // Few tiles and many k-blocks: clusters of `split` CTAs share a tile's k-blocks and merge their sums through distributed
-  // shared memory, 2.6 to 2.9 us more for two cluster barriers and the merge.  64 x 5120 -> 640: 14.3 -> 6.3 us, 256 x 5120
-  // -> 1536: 14.7 -> 8.6, 40 x 1536 -> 1536: 6.4 -> 6.0; 512 x 2048 -> 2048 stays whole (7.97 against 8.54).  As
-  // many clusters as run at once: of four or eight CTAs that is about four fifths of the chip.
+  // Few tiles and many k-blocks: clusters of `split` CTAs share a tile's k-blocks and merge their sums through
+  // distributed shared memory, 2.6 to 2.9 us more for two cluster barriers and the merge.  64 x 5120 -> 640: 14.3 ->
+  // 6.3 us, 256 x 5120 -> 1536: 14.7 -> 8.6, 40 x 1536 -> 1536: 6.4 -> 6.0; 512 x 2048 -> 2048 stays whole (7.97
+  // against 8.54).  As many clusters as run at once: of four or eight CTAs that is taken as four fifths of the chip
+  // (any more would run later: an estimate, not a limit).
   int split = 1;
   for (const int c : {2, 4, 8}) {
     const int64_t tiles = m_tiles * (Dout / 128);
