@@ -510,7 +510,8 @@ ISPA_API size_t ispa_ls_solve_workspace_size(int32_t dim, int32_t d_out);
  * M = G + lambda I a diagonal near 1 and X's columns one size.  So row i of X W is off by at most
  * dim 2^-54 sqrt(M_ii) max_j (sqrt(S_jj) |W_jk|), where fp64 arithmetic has
  * dim 2^-53 sum_j |X_ij W_jk|, and what the factorisation and the solves lose is a perturbation of
- * M_ij small against sqrt(M_ii M_jj), as in an fp64 Cholesky solve.
+ * M_ij small against sqrt(M_ii M_jj), as in an fp64 Cholesky solve.  Errors are relative to the
+ * largest sqrt(M_ii) |dW_ik| of a column k, not to each of them.
  * Synchronises `stream`.  Errors: ISPA_ERR_NOT_SPD if a Cholesky pivot is not
  * positive (dW and eps are then meaningless); ISPA_ERR_TIMEOUT if a device wait ran out.
  */
