@@ -805,6 +805,61 @@ static int gram_grid(int64_t total, int64_t len, int sms, int flush) {
   return 21 * steps * sms < 20 * (total + flush * sms) ? static_cast<int>(passes * m) : sms;
 }
 
+// Steps of the CTA that has most of them when gram_wide_kernel runs on `grid` CTAs: whole tiles in waves, then an equal
+// share of the rest; each tile or part of one is flushed at the cost of `flush` steps.
+static int64_t wide_cost(const WideParams& p, int grid, int flush) {
+  int64_t fixed = 0, tail = 0, left[3], len[3];
+  for (int k = 0; k < 3; ++k) {
+    len[k] = static_cast<int64_t>(p.passes[k]) * p.n_ktiles;
+    left[k] = p.U[k] % grid;
+    fixed += p.U[k] / grid * (len[k] + flush);
+    tail += left[k] * len[k];
+  }
+  int64_t most = 0, pos = 0, tile_end = 0;
+  for (int i = 0, k = 0; i < grid; ++i) {
+    const int64_t end = tail * (i + 1) / grid;
+    int64_t cost = end - pos;
+    while (pos < end) {
+      if (pos == tile_end) {
+        while (left[k] == 0) ++k;
+        --left[k];
+        tile_end += len[k];
+      }
+      cost += flush;
+      pos = end < tile_end ? end : tile_end;
+    }
+    most = cost > most ? cost : most;
+  }
+  return fixed + most;
+}
+
+// With more tile passes than SMs, a call of up to 1024 tokens is bound by its flushes, and one CTA per SM cuts most
+// tiles in two.  So the grids that don't: the most CTAs that take the same whole number of passes each, or else as many
+// as make full waves of the G and S or of the X tiles, if that saves 6 % of the longest CTA's steps.  us, one CTA per
+// SM against this (two calls and the reset): D 2048 exact, 500 tokens 71.8 -> 63.9 (136 CTAs); D 2560, 500 tokens
+// 89.6 -> 82.1 (105); D 4096 exact, 84 tokens 202 -> 175 (132); D 3840 exact, 84 tokens 165 -> 158 (120).  Above 1024
+// tokens the steps count: D 3072, 1500 tokens 153 us on 152 CTAs, 157 on 150.
+static int wide_grid(const WideParams& p, int64_t passes, int sms, int flush) {
+  if (p.n_ktiles > 16) return sms;
+  const int64_t all = wide_cost(p, sms, flush);
+  auto saves = [&](int grid) { return 106 * wide_cost(p, grid, flush) < 100 * all; };
+  int64_t k = (passes + sms - 1) / sms;
+  while (k <= 24 && passes % k != 0) ++k;
+  if (passes % k == 0 && passes / k < sms && saves(static_cast<int>(passes / k))) return static_cast<int>(passes / k);
+  int best = sms;
+  int64_t best_cost = all;
+  for (int j = 0; j < 2; ++j) {
+    const int waves = (p.U[j] + sms - 1) / sms, grid = (p.U[j] + waves - 1) / waves;
+    if (!saves(grid)) continue;
+    const int64_t cost = wide_cost(p, grid, flush);
+    if (cost < best_cost) {
+      best = grid;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
 static cudaError_t launch_gram_wide(int32_t D, int64_t T, int form, const void* op0, const void* op1,
                                     const void* op2, const float* unscale, float* gram, int* status,
                                     uint64_t wait_limit_ns, uint32_t* hb, cudaStream_t s) {
@@ -844,7 +899,8 @@ static cudaError_t launch_gram_wide(int32_t D, int64_t T, int form, const void* 
   int64_t total = 0;
   for (int k = 0; k < 3; ++k) total += static_cast<int64_t>(p.U[k]) * passes[k] * p.n_ktiles;
   if (total > INT32_MAX) return cudaErrorInvalidValue;
-  const int grid = gram_grid(total, p.n_ktiles, sms, 9);
+  const int64_t n_passes = total / p.n_ktiles;
+  const int grid = n_passes > sms ? wide_grid(p, n_passes, sms, 9) : gram_grid(total, p.n_ktiles, sms, 9);
   p.tail_total = 0;
   for (int k = 0; k < 3; ++k) {
     p.waves[k] = p.U[k] / grid;
